@@ -641,14 +641,14 @@ static int launch_run(sp_mc *h, u64 n_photons, u64 seed, u64 pid_begin, const u6
     const bool field = h->field != 0;
     if (smem > 48 * 1024) {
         CUDA_TRY(cudaFuncSetAttribute(f64 ? kernel_f64(field, h->mirror != 0)
-                                          : kernel_f32(field, h->mirror != 0, h->variant),
+                                          : kernel_f32(field, h->mirror != 0, h->variant, h->n_rec > 0),
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     }
     int blocks = h->blocks_opt;
     if (blocks <= 0) {
         int per_sm = 0;
         CUDA_TRY(f64 ? occupancy_f64(field, h->mirror != 0, h->threads, smem, &per_sm)
-                     : occupancy_f32(field, h->mirror != 0, h->variant, h->threads, smem, &per_sm));
+                     : occupancy_f32(field, h->mirror != 0, h->variant, h->n_rec > 0, h->threads, smem, &per_sm));
         if (per_sm < 1) return fail(SP_ECUDA, "transport kernel cannot be resident with %zu B smem", smem);
         blocks = per_sm * h->sm_count;
     }
@@ -967,7 +967,7 @@ extern "C" int sp_mc_simulate_noalloc(const uint8_t *d_mask, int nx, int ny, int
     tmp.porosity = porosity;
     set_bin_mul(&tmp);
     int per_sm = 0;
-    if (occupancy_f32(false, false, tmp.variant, tmp.threads, 0, &per_sm) != cudaSuccess || per_sm < 1)
+    if (occupancy_f32(false, false, tmp.variant, false, tmp.threads, 0, &per_sm) != cudaSuccess || per_sm < 1)
         return fail(SP_ECUDA, "CUDA error");
 
     TransportParams p{};

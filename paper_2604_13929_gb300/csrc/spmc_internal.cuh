@@ -63,6 +63,10 @@ struct TransportParams {
     int nbx, nby, nbz;             // bricks per axis (ceil(n/4))
     int smem_bricks;               // leading bricks (z-major) staged per CTA
     u32 key0, key1;                // Philox key = seed
+    u32 rk[20];                    // Philox round keys (FP32 streamlined kernel)
+    u32 first;                     // photons assigned to each warp at the start (streamlined kernel)
+    u32 claim;                     // photons of a later claim, from index claim_base on
+    u64 claim_base;
     u64 pid_begin, n_photons;
     const u64 *pid_begin_dev;      // if set, the first photon id is read here (graph replays)
     double mus, mua, g;
@@ -111,9 +115,18 @@ struct BatchParams {
     u32 chunk;                      // photons per chunk (streamlined kernel)
     u64 *next;                      // claim counter, zeroed before each launch
     u32 key0, key1;                 // Philox key = seed (shared by all problems)
+    u32 rk[20];                     // its round keys (streamlined kernel)
     int compact_k;
     int steps_per_pass;
 };
+
+// Philox round keys of a seed: round r uses key + r times the Weyl constants.
+inline void philox_round_keys(u32 k0, u32 k1, u32 (&rk)[20]) {
+    for (u32 r = 0; r < 10; ++r) {
+        rk[2 * r] = k0 + r * 0x9E3779B9u;
+        rk[2 * r + 1] = k1 + r * 0xBB67AE85u;
+    }
+}
 
 // Launch choices of the FP32 path beyond TransportParams: which kernel.
 struct LaunchExtras {
@@ -121,17 +134,17 @@ struct LaunchExtras {
 };
 
 // Launch helpers (defined in the per-precision translation units).
-cudaError_t launch_transport_f32(const TransportParams &p, bool field, int blocks, int threads,
+cudaError_t launch_transport_f32(TransportParams p, bool field, int blocks, int threads,
                                  size_t smem, cudaStream_t s, const LaunchExtras &e);
 cudaError_t launch_transport_f64(const TransportParams &p, bool field, int blocks, int threads,
                                  size_t smem, cudaStream_t s);
-cudaError_t occupancy_f32(bool field, bool mirror, int variant, int threads, size_t smem,
+cudaError_t occupancy_f32(bool field, bool mirror, int variant, bool rec, int threads, size_t smem,
                           int *blocks_per_sm);
-cudaError_t launch_transport_batch(const BatchParams &b, int variant, bool mirror, int blocks,
+cudaError_t launch_transport_batch(BatchParams b, int variant, bool mirror, int blocks,
                                    int threads, cudaStream_t s);
 cudaError_t occupancy_batch(int variant, bool mirror, int threads, int *blocks_per_sm);
 cudaError_t occupancy_f64(bool field, bool mirror, int threads, size_t smem, int *blocks_per_sm);
-const void *kernel_f32(bool field, bool mirror, int variant);
+const void *kernel_f32(bool field, bool mirror, int variant, bool rec);
 const void *kernel_f64(bool field, bool mirror);
 
 }  // namespace spmc

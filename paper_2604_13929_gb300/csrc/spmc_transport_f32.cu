@@ -7,14 +7,20 @@ namespace spmc {
 
 namespace {
 
-template <bool kField, bool kMirror>
-const void *fast_ptr() {
-    return reinterpret_cast<const void *>(&transport_f32_kernel<kField, kMirror, false>);
+using FastKernel = void (*)(TransportParams, BatchParams);
+
+// The streamlined kernel of a launch.  Runs that record photons take the
+// builds with unwrapped positions and per-photon counts (mirror faces decided
+// at run time there).
+FastKernel fast_kernel(bool field, bool mirror, bool rec) {
+    if (rec) return field ? &transport_f32_kernel<true, true, false, true> : &transport_f32_kernel<false, true, false, true>;
+    if (mirror)
+        return field ? &transport_f32_kernel<true, true, false, false> : &transport_f32_kernel<false, true, false, false>;
+    return field ? &transport_f32_kernel<true, false, false, false> : &transport_f32_kernel<false, false, false, false>;
 }
 
-const void *fast_kernel(bool field, bool mirror) {
-    if (mirror) return field ? fast_ptr<true, true>() : fast_ptr<false, true>();
-    return field ? fast_ptr<true, false>() : fast_ptr<false, false>();
+FastKernel fast_batch_kernel(bool mirror) {
+    return mirror ? &transport_f32_kernel<true, true, true, false> : &transport_f32_kernel<true, false, true, false>;
 }
 
 // per-warp tallies of the streamlined batched kernel (dynamic shared memory)
@@ -22,47 +28,49 @@ size_t batch_smem(int threads) { return (size_t)(threads / 32) * sizeof(SmemTall
 
 const void *batch_kernel(int variant, bool mirror) {
     if (variant == 0) return reinterpret_cast<const void *>(&transport_kernel<float, true, true, true>);
-    return mirror ? reinterpret_cast<const void *>(&transport_f32_kernel<true, true, true>)
-                  : reinterpret_cast<const void *>(&transport_f32_kernel<true, false, true>);
+    return reinterpret_cast<const void *>(fast_batch_kernel(mirror));
 }
 
 }  // namespace
 
-const void *kernel_f32(bool field, bool mirror, int variant) {
-    return variant == 0 ? kernel_ptr<float>(field, mirror) : fast_kernel(field, mirror);
+const void *kernel_f32(bool field, bool mirror, int variant, bool rec) {
+    return variant == 0 ? kernel_ptr<float>(field, mirror)
+                        : reinterpret_cast<const void *>(fast_kernel(field, mirror, rec));
 }
 
-cudaError_t launch_transport_f32(const TransportParams &p, bool field, int blocks, int threads,
+cudaError_t launch_transport_f32(TransportParams p, bool field, int blocks, int threads,
                                  size_t smem, cudaStream_t s, const LaunchExtras &e) {
     if (e.variant == 0) return launch_transport<float>(p, field, blocks, threads, smem, s);
+    philox_round_keys(p.key0, p.key1, p.rk);
+    // Photons by warp: 32 at the start (fewer, down to 8, when there are not
+    // enough for every warp), then claims of 32 that shrink with the photons
+    // per warp so that the last claims stay balanced.
+    const u64 warps = (u64)blocks * (u64)(threads / 32), per_warp = p.n_photons / warps;
+    p.first = per_warp >= 32 ? 32u : (per_warp < 8 ? 8u : (u32)per_warp);
+    p.claim_base = warps * p.first;
+    p.claim = per_warp >= 256 ? 32u : (per_warp < 64 ? 8u : (u32)(per_warp / 8));
     const BatchParams none{};
-    if (p.mirror) {
-        if (field) transport_f32_kernel<true, true, false><<<blocks, threads, smem, s>>>(p, none);
-        else transport_f32_kernel<false, true, false><<<blocks, threads, smem, s>>>(p, none);
-    } else {
-        if (field) transport_f32_kernel<true, false, false><<<blocks, threads, smem, s>>>(p, none);
-        else transport_f32_kernel<false, false, false><<<blocks, threads, smem, s>>>(p, none);
-    }
+    fast_kernel(field, p.mirror != 0, p.n_rec > 0)<<<blocks, threads, smem, s>>>(p, none);
     return cudaGetLastError();
 }
 
-cudaError_t occupancy_f32(bool field, bool mirror, int variant, int threads, size_t smem,
+cudaError_t occupancy_f32(bool field, bool mirror, int variant, bool rec, int threads, size_t smem,
                           int *blocks_per_sm) {
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kernel_f32(field, mirror, variant),
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kernel_f32(field, mirror, variant, rec),
                                                          threads, smem);
 }
 
 // Batched launches: variant 0 the generic kernel (lanes of a warp carry
 // photons of different problems), 1 the streamlined kernel (chunks of one
 // problem per warp).  mirror: some problem has mirror lateral faces.
-cudaError_t launch_transport_batch(const BatchParams &b, int variant, bool mirror, int blocks,
+cudaError_t launch_transport_batch(BatchParams b, int variant, bool mirror, int blocks,
                                    int threads, cudaStream_t s) {
     TransportParams p{};
     p.compact_k = b.compact_k;
+    philox_round_keys(b.key0, b.key1, b.rk);
     const size_t smem = variant == 0 ? 0 : batch_smem(threads);
     if (variant == 0) transport_kernel<float, true, true, true><<<blocks, threads, 0, s>>>(p, b);
-    else if (mirror) transport_f32_kernel<true, true, true><<<blocks, threads, smem, s>>>(p, b);
-    else transport_f32_kernel<true, false, true><<<blocks, threads, smem, s>>>(p, b);
+    else fast_batch_kernel(mirror)<<<blocks, threads, smem, s>>>(p, b);
     return cudaGetLastError();
 }
 

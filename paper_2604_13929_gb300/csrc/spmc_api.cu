@@ -124,9 +124,11 @@ static void set_bin_mul(sp_mc *h) {
 // FP32 copies of the optics and limits of a launch (computed on the host so
 // FP32 kernels never convert doubles inside their loop).
 static void fill_f32(const sp_mc *h, double s_max, TransportParams::F32 &f, int &hg_iso,
-                     int &small_x) {
+                     int &small_x, int &plain) {
     hg_iso = std::fabs(h->g) < 1e-6;
     small_x = h->mua * 1.7320508075688772 <= 0.1;
+    // photons start at weight 1 and roulette lifts a weight below rr_weight rr_mult-fold
+    plain = small_x && h->rr_weight * h->rr_mult <= 1.0;
     f.mus = (float)h->mus;
     f.mua = (float)h->mua;
     f.inv_mus = h->mus > 0 ? (float)(1.0 / h->mus) : 0.0f;
@@ -627,6 +629,10 @@ int sp_mc_get_option(const sp_mc_t *h, int key, double *value) {
     }
 }
 
+// Runs that record photons and volumes whose voxel addresses need more than
+// 32 bits take the FP32 kernel's general builds.
+static bool wide_build(const sp_mc *h) { return h->n_rec > 0 || h->n_field > 0xffffffffull; }
+
 // One single-problem transport launch of n_photons from photon id pid_begin
 // (or from *pid_begin_dev when it is set), stream-ordered and capturable.
 static int launch_run(sp_mc *h, u64 n_photons, u64 seed, u64 pid_begin, const u64 *pid_begin_dev,
@@ -636,19 +642,26 @@ static int launch_run(sp_mc *h, u64 n_photons, u64 seed, u64 pid_begin, const u6
     int smem_bricks = h->smem_bricks_opt;
     if (smem_bricks < 0) smem_bricks = (int)std::min<u64>(n_bricks, 12288);   // auto: 96 KiB
     smem_bricks = (int)std::min<u64>((u64)smem_bricks, n_bricks);
-    const size_t smem = (size_t)smem_bricks * sizeof(u64);
     const bool f64 = h->precision == 64;
     const bool field = h->field != 0;
+    const size_t extra = f64 ? 0 : smem_f32(field, h->variant, h->threads);
+    constexpr size_t kMaxSmem = 227 * 1024;
+    // the FP32 kernel's own shared memory comes out of a slab that would
+    // otherwise fill an SM's (staging more or fewer bricks changes no result)
+    if (extra && (size_t)smem_bricks * sizeof(u64) + 4352 <= kMaxSmem)
+        smem_bricks = (int)std::min<size_t>((size_t)smem_bricks, (kMaxSmem - extra) / sizeof(u64));
+    const size_t smem = (size_t)smem_bricks * sizeof(u64) + extra;
+    const bool wide = wide_build(h);
     if (smem > 48 * 1024) {
         CUDA_TRY(cudaFuncSetAttribute(f64 ? kernel_f64(field, h->mirror != 0)
-                                          : kernel_f32(field, h->mirror != 0, h->variant, h->n_rec > 0),
+                                          : kernel_f32(field, h->mirror != 0, h->variant, wide),
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     }
     int blocks = h->blocks_opt;
     if (blocks <= 0) {
         int per_sm = 0;
         CUDA_TRY(f64 ? occupancy_f64(field, h->mirror != 0, h->threads, smem, &per_sm)
-                     : occupancy_f32(field, h->mirror != 0, h->variant, h->n_rec > 0, h->threads, smem, &per_sm));
+                     : occupancy_f32(field, h->mirror != 0, h->variant, wide, h->threads, smem, &per_sm));
         if (per_sm < 1) return fail(SP_ECUDA, "transport kernel cannot be resident with %zu B smem", smem);
         blocks = per_sm * h->sm_count;
     }
@@ -680,10 +693,11 @@ static int launch_run(sp_mc *h, u64 n_photons, u64 seed, u64 pid_begin, const u6
     p.steps_per_pass = h->steps_per_pass;
     p.bin_mul = h->bin_mul;
     p.bin_exact = h->bin_exact;
-    fill_f32(h, p.s_max, p.f32, p.hg_iso, p.small_x);
+    fill_f32(h, p.s_max, p.f32, p.hg_iso, p.small_x, p.plain);
 
     LaunchExtras ex;
     ex.variant = h->variant;
+    ex.wide = wide;
     CUDA_TRY(cudaMemsetAsync(&h->d_tal->next, 0, sizeof(u64), s));
     CUDA_TRY(f64 ? launch_transport_f64(p, field, blocks, h->threads, smem, s)
                  : launch_transport_f32(p, field, blocks, h->threads, smem, s, ex));
@@ -967,7 +981,8 @@ extern "C" int sp_mc_simulate_noalloc(const uint8_t *d_mask, int nx, int ny, int
     tmp.porosity = porosity;
     set_bin_mul(&tmp);
     int per_sm = 0;
-    if (occupancy_f32(false, false, tmp.variant, false, tmp.threads, 0, &per_sm) != cudaSuccess || per_sm < 1)
+    const size_t smem = smem_f32(false, tmp.variant, tmp.threads);
+    if (occupancy_f32(false, false, tmp.variant, false, tmp.threads, smem, &per_sm) != cudaSuccess || per_sm < 1)
         return fail(SP_ECUDA, "CUDA error");
 
     TransportParams p{};
@@ -991,11 +1006,11 @@ extern "C" int sp_mc_simulate_noalloc(const uint8_t *d_mask, int nx, int ny, int
     p.steps_per_pass = tmp.steps_per_pass;
     p.bin_mul = tmp.bin_mul;
     p.bin_exact = tmp.bin_exact;
-    fill_f32(&tmp, p.s_max, p.f32, p.hg_iso, p.small_x);
+    fill_f32(&tmp, p.s_max, p.f32, p.hg_iso, p.small_x, p.plain);
     LaunchExtras ex;
     ex.variant = tmp.variant;
 
-    if (n_photons > 0 && launch_transport_f32(p, false, per_sm * sms, tmp.threads, 0, s, ex) != cudaSuccess)
+    if (n_photons > 0 && launch_transport_f32(p, false, per_sm * sms, tmp.threads, smem, s, ex) != cudaSuccess)
         return fail(SP_ECUDA, "CUDA error");
     finalize_kernel<<<1, kNBin, 0, s>>>(tal, nullptr, bin_count, nx, ny, nz, porosity, d_result);
     u32 flags = 0;
@@ -1244,10 +1259,11 @@ static int batch_launch(sp_mc_batch *b, u64 total, cudaStream_t s) {
     return SP_OK;
 }
 
-// Whether any problem has mirror lateral faces (selects the batched kernel).
+// Whether any problem has mirror lateral faces or 64-bit voxel addresses
+// (selects the batched kernel's general build).
 static void refresh_mirror(sp_mc_batch *b) {
     b->any_mirror = false;
-    for (const sp_mc *h : b->h) b->any_mirror = b->any_mirror || h->mirror != 0;
+    for (const sp_mc *h : b->h) b->any_mirror = b->any_mirror || h->mirror != 0 || wide_build(h);
 }
 
 extern "C" int sp_mc_batch_run(sp_mc_batch_t *b, const uint64_t *n_photons, uint64_t seed,
@@ -1285,7 +1301,7 @@ extern "C" int sp_mc_batch_run(sp_mc_batch_t *b, const uint64_t *n_photons, uint
             chunk_begin += (n_photons[i] + b->chunk - 1) / b->chunk;
             const u64 lim = iter_limit(h);
             t.iter_limit = lim > 0xffffffffull ? 0xffffffffu : (u32)lim;
-            fill_f32(h, path_cap(h), t.f32, t.hg_iso, t.small_x);
+            fill_f32(h, path_cap(h), t.f32, t.hg_iso, t.small_x, t.plain);
             t.mirror = h->mirror;
             CUDA_TRY(cudaMemsetAsync(&h->d_tal->next, 0, sizeof(u64), s));
         }

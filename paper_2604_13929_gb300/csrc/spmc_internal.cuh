@@ -63,7 +63,6 @@ struct TransportParams {
     int nbx, nby, nbz;             // bricks per axis (ceil(n/4))
     int smem_bricks;               // leading bricks (z-major) staged per CTA
     u32 key0, key1;                // Philox key = seed
-    u32 rk[20];                    // Philox round keys (FP32 streamlined kernel)
     u32 first;                     // photons assigned to each warp at the start (streamlined kernel)
     u32 claim;                     // photons of a later claim, from index claim_base on
     u64 claim_base;
@@ -76,6 +75,7 @@ struct TransportParams {
     int hg_iso;                    // |g| < 1e-6: isotropic scattering
     int mirror;                    // lateral faces: 0 periodic, 1 specular mirrors
     int small_x;                   // mu_a * sqrt(3) <= 0.1: Taylor branch for 1 - exp(-x)
+    int plain;                     // small_x and no weight above 1: the FP32 kernel's plain step applies
     int steps_per_pass;            // FP32 kernel: voxel steps per pass of the warp
     u32 bin_mul;                   // depth bin = umulhi(64 iz, bin_mul) when bin_exact
     int bin_exact;
@@ -103,7 +103,7 @@ struct BatchProblem {
     u64 pid_begin, n_photons, offset;
     u64 chunk_begin;
     u32 iter_limit;
-    int hg_iso, small_x, mirror;
+    int hg_iso, small_x, plain, mirror;
     TransportParams::F32 f32;
 };
 
@@ -115,22 +115,14 @@ struct BatchParams {
     u32 chunk;                      // photons per chunk (streamlined kernel)
     u64 *next;                      // claim counter, zeroed before each launch
     u32 key0, key1;                 // Philox key = seed (shared by all problems)
-    u32 rk[20];                     // its round keys (streamlined kernel)
     int compact_k;
     int steps_per_pass;
 };
 
-// Philox round keys of a seed: round r uses key + r times the Weyl constants.
-inline void philox_round_keys(u32 k0, u32 k1, u32 (&rk)[20]) {
-    for (u32 r = 0; r < 10; ++r) {
-        rk[2 * r] = k0 + r * 0x9E3779B9u;
-        rk[2 * r + 1] = k1 + r * 0xBB67AE85u;
-    }
-}
-
 // Launch choices of the FP32 path beyond TransportParams: which kernel.
 struct LaunchExtras {
     int variant = 1;               // 0 generic template kernel, 1 streamlined FP32 kernel
+    bool wide = false;             // streamlined kernel: photon records or 64-bit voxel addresses
 };
 
 // Launch helpers (defined in the per-precision translation units).
@@ -138,13 +130,16 @@ cudaError_t launch_transport_f32(TransportParams p, bool field, int blocks, int 
                                  size_t smem, cudaStream_t s, const LaunchExtras &e);
 cudaError_t launch_transport_f64(const TransportParams &p, bool field, int blocks, int threads,
                                  size_t smem, cudaStream_t s);
-cudaError_t occupancy_f32(bool field, bool mirror, int variant, bool rec, int threads, size_t smem,
+// Dynamic shared memory of the FP32 kernel beside the staged bricks; part of
+// `smem` in the launch and the occupancy query.
+size_t smem_f32(bool field, int variant, int threads);
+cudaError_t occupancy_f32(bool field, bool mirror, int variant, bool wide, int threads, size_t smem,
                           int *blocks_per_sm);
 cudaError_t launch_transport_batch(BatchParams b, int variant, bool mirror, int blocks,
                                    int threads, cudaStream_t s);
 cudaError_t occupancy_batch(int variant, bool mirror, int threads, int *blocks_per_sm);
 cudaError_t occupancy_f64(bool field, bool mirror, int threads, size_t smem, int *blocks_per_sm);
-const void *kernel_f32(bool field, bool mirror, int variant, bool rec);
+const void *kernel_f32(bool field, bool mirror, int variant, bool wide);
 const void *kernel_f64(bool field, bool mirror);
 
 }  // namespace spmc

@@ -9,11 +9,12 @@ namespace {
 
 using FastKernel = void (*)(TransportParams, BatchParams);
 
-// The streamlined kernel of a launch.  Runs that record photons take the
-// builds with unwrapped positions and per-photon counts (mirror faces decided
-// at run time there).
-FastKernel fast_kernel(bool field, bool mirror, bool rec) {
-    if (rec) return field ? &transport_f32_kernel<true, true, false, true> : &transport_f32_kernel<false, true, false, true>;
+// The streamlined kernel of a launch.  Runs that record photons and volumes
+// of 2^26 bricks and more take the builds with 64-bit voxel addresses,
+// unwrapped positions and per-photon counts (mirror faces decided at run time
+// there).
+FastKernel fast_kernel(bool field, bool mirror, bool wide) {
+    if (wide) return field ? &transport_f32_kernel<true, true, false, true> : &transport_f32_kernel<false, true, false, true>;
     if (mirror)
         return field ? &transport_f32_kernel<true, true, false, false> : &transport_f32_kernel<false, true, false, false>;
     return field ? &transport_f32_kernel<true, false, false, false> : &transport_f32_kernel<false, false, false, false>;
@@ -23,8 +24,7 @@ FastKernel fast_batch_kernel(bool mirror) {
     return mirror ? &transport_f32_kernel<true, true, true, false> : &transport_f32_kernel<true, false, true, false>;
 }
 
-// per-warp tallies of the streamlined batched kernel (dynamic shared memory)
-size_t batch_smem(int threads) { return (size_t)(threads / 32) * sizeof(SmemTallies); }
+size_t batch_smem(int threads) { return f32_smem(true, true, threads); }
 
 const void *batch_kernel(int variant, bool mirror) {
     if (variant == 0) return reinterpret_cast<const void *>(&transport_kernel<float, true, true, true>);
@@ -33,15 +33,18 @@ const void *batch_kernel(int variant, bool mirror) {
 
 }  // namespace
 
-const void *kernel_f32(bool field, bool mirror, int variant, bool rec) {
+const void *kernel_f32(bool field, bool mirror, int variant, bool wide) {
     return variant == 0 ? kernel_ptr<float>(field, mirror)
-                        : reinterpret_cast<const void *>(fast_kernel(field, mirror, rec));
+                        : reinterpret_cast<const void *>(fast_kernel(field, mirror, wide));
+}
+
+size_t smem_f32(bool field, int variant, int threads) {
+    return variant == 0 ? 0 : f32_smem(field, false, threads);
 }
 
 cudaError_t launch_transport_f32(TransportParams p, bool field, int blocks, int threads,
                                  size_t smem, cudaStream_t s, const LaunchExtras &e) {
     if (e.variant == 0) return launch_transport<float>(p, field, blocks, threads, smem, s);
-    philox_round_keys(p.key0, p.key1, p.rk);
     // Photons by warp: 32 at the start (fewer, down to 8, when there are not
     // enough for every warp), then claims of 32 that shrink with the photons
     // per warp so that the last claims stay balanced.
@@ -50,13 +53,13 @@ cudaError_t launch_transport_f32(TransportParams p, bool field, int blocks, int 
     p.claim_base = warps * p.first;
     p.claim = per_warp >= 256 ? 32u : (per_warp < 64 ? 8u : (u32)(per_warp / 8));
     const BatchParams none{};
-    fast_kernel(field, p.mirror != 0, p.n_rec > 0)<<<blocks, threads, smem, s>>>(p, none);
+    fast_kernel(field, p.mirror != 0, e.wide)<<<blocks, threads, smem, s>>>(p, none);
     return cudaGetLastError();
 }
 
-cudaError_t occupancy_f32(bool field, bool mirror, int variant, bool rec, int threads, size_t smem,
+cudaError_t occupancy_f32(bool field, bool mirror, int variant, bool wide, int threads, size_t smem,
                           int *blocks_per_sm) {
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kernel_f32(field, mirror, variant, rec),
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kernel_f32(field, mirror, variant, wide),
                                                          threads, smem);
 }
 
@@ -67,7 +70,6 @@ cudaError_t launch_transport_batch(BatchParams b, int variant, bool mirror, int 
                                    int threads, cudaStream_t s) {
     TransportParams p{};
     p.compact_k = b.compact_k;
-    philox_round_keys(b.key0, b.key1, b.rk);
     const size_t smem = variant == 0 ? 0 : batch_smem(threads);
     if (variant == 0) transport_kernel<float, true, true, true><<<blocks, threads, 0, s>>>(p, b);
     else fast_batch_kernel(mirror)<<<blocks, threads, smem, s>>>(p, b);

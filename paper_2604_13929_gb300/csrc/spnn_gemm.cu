@@ -1,8 +1,8 @@
 // spnn_gemm.cu -- the tensor-core GEMM kernels of the surrogate: rows_kernel
-// (forward and input-gradient layers), wgrad_kernel and wgrad_halo_kernel
-// (weight gradients).
+// and slab_kernel (forward and input-gradient layers), wgrad_kernel and
+// wgrad_halo_kernel (weight gradients).
 //
-// All are warp-specialised, 192 threads:
+// All are warp-specialised, 192 threads (slab_kernel 320):
 //   warp 0      TMA producer: fills a ring of shared-memory stages,
 //   warp 1      allocates TMEM and issues tcgen05.mma,
 //   warps 2..5  epilogue: tcgen05.ld of the FP32 accumulators, fused
@@ -142,6 +142,301 @@ __device__ __forceinline__ void tile_origin_u32(const TileGrid& g, uint32_t t, i
     q = t / (uint32_t)g.nz;
     z0 = (int)(t - q * (uint32_t)g.nz) * g.bz;
     b0 = (int)q * g.bb;
+}
+
+// Epilogue of 16 accumulator columns of one voxel: bias, residual, ReLU or
+// ReLU-derivative mask, two 16-byte BF16 stores (channels ch0 .. ch0 + 15 at
+// off); adds the rounded outputs' dot product with head_w (if given) to head.
+__device__ __forceinline__ void emit16(const EpiDest& d, const uint32_t (&v)[16], int ch0, long long off,
+                                       const float* head_w, float& head) {
+    float f[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) f[i] = __uint_as_float(v[i]);
+    if (d.bias) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) f[i] += d.bias[ch0 + i];
+    }
+    if (d.addend) {
+        float a[16];
+        load16_planes(d.addend + off, d.plane, a);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) f[i] += a[i];
+    }
+    if (d.relu) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) f[i] = fmaxf(f[i], 0.f);
+    }
+    if (d.mask) {
+        float mk[16];
+        load16_planes(d.mask + off, d.plane, mk);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) f[i] = (mk[i] > 0.f) ? f[i] : 0.f;
+    }
+    uint4 w[2];
+    __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(w);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) h[i] = __floats2bfloat162_rn(f[2 * i], f[2 * i + 1]);
+    *reinterpret_cast<uint4*>(d.out + off) = w[0];
+    *reinterpret_cast<uint4*>(d.out + off + d.plane) = w[1];
+    if (head_w) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float2 rb = __bfloat1622float2(h[i]);
+            head += rb.x * head_w[ch0 + 2 * i] + rb.y * head_w[ch0 + 2 * i + 1];
+        }
+    }
+}
+
+// The MMAs of one stage (ZC input planes) of the z-walk, as one straight run of
+// 3 ZC instructions: an input plane is only three MMAs of 48 to 96 cycles, and a
+// loop that works out its operands takes a lone warp about 300 cycles a plane.
+// So everything but the stage's bases is a compile-time constant: N output
+// channels, START / END (the stage holds the box's first / last input planes,
+// which feed fewer output planes), FIRST (the first K-step: the newest output
+// plane of an MMA, its last N columns, is overwritten, in an MMA of its own).
+// a: descriptor low word of the stage's first plane, zrow / row: 16-byte units
+// of a z-plane and a y-row; b: low word of the K-step's weights; col: columns
+// of output plane z - 1 of the stage's first input plane z (0 with START).
+template <int N, int ZC, bool START, bool END, bool FIRST>
+__device__ __forceinline__ void slab_stage(uint32_t col, uint32_t a, uint32_t a_hi, uint32_t zrow, uint32_t row,
+                                           uint32_t b, uint32_t b_hi) {
+#pragma unroll
+    for (int zi = 0; zi < ZC; ++zi) {
+        // output planes j0 <= j < j1 of (z - 1, z, z + 1)
+        const int j0 = START ? (zi == 0 ? 2 : (zi == 1 ? 1 : 0)) : 0;
+        const int j1 = END ? (zi == ZC - 1 ? 1 : (zi == ZC - 2 ? 2 : 3)) : 3;
+        const int cnt = j1 - j0;
+        const uint32_t c = col + (uint32_t)((START ? (zi < 2 ? 0 : zi - 2) : zi) * N);
+        const uint32_t az = a + (uint32_t)zi * zrow, bz = b + (uint32_t)(j0 * N);
+        if (FIRST && j1 == 3) {
+            if (cnt > 1) umma_bf16_lo<1>(c, az, a_hi, bz, b_hi, idesc_bf16(128, (cnt - 1) * N, 0, 0));
+            umma_bf16_lo<0>(c + (uint32_t)((cnt - 1) * N), az, a_hi, bz + (uint32_t)((cnt - 1) * N), b_hi,
+                            idesc_bf16(128, N, 0, 0));
+        } else {
+            umma_bf16_lo<1>(c, az, a_hi, bz, b_hi, idesc_bf16(128, cnt * N, 0, 0));
+        }
+        umma_bf16_lo<1>(c, az + row, a_hi, bz + 3u * N, b_hi, idesc_bf16(128, cnt * N, 0, 0));
+        umma_bf16_lo<1>(c, az + 2u * row, a_hi, bz + 6u * N, b_hi, idesc_bf16(128, cnt * N, 0, 0));
+    }
+}
+
+// MMA warp of slab_kernel: the whole warp walks the K-steps, one elected lane
+// issues (see rows_kernel).  ZST stages of ZC input planes per K-step.
+template <int N, int ZC, int ZST>
+__device__ __forceinline__ void slab_issue(const SlabParams& p, uint32_t bar0, uint32_t acc_full, uint32_t acc_empty,
+                                           uint32_t w_full, uint32_t wbase, uint32_t sbase, uint32_t tmem) {
+    const bool leader = elect_one();
+    const int S = p.stages, ksteps = 3 * (p.kc_total / 2);
+    const uint32_t acc_cols = (uint32_t)p.zp * N;
+    const uint32_t row = (uint32_t)p.g.bx, zrow = row * (uint32_t)(p.g.by + 2);
+    const uint64_t ad = smem_desc(sbase, zrow * 16u * ZC, 128), bd = smem_desc(wbase, 9u * N * 16u, 128);
+    const uint32_t a_hi = (uint32_t)(ad >> 32), b_hi = (uint32_t)(bd >> 32), stage_u = p.stage_bytes / 16u;
+    auto wait = [&](uint32_t bar, uint32_t parity) -> bool {
+        const bool ok = __all_sync(0xffffffffu, mbar_wait(bar, parity, kWaitLimitNs));
+        if (!ok && leader) atomicOr(p.err, ERR_TIMEOUT);
+        return ok;
+    };
+    if (!wait(w_full, 0)) return;
+    Ring q;
+    uint32_t it = 0;
+    for (int t = blockIdx.x; t < p.tiles; t += gridDim.x, ++it) {
+        const uint32_t buf = it & 1u, use = it >> 1;
+        if (use > 0 && !wait(acc_empty + 8u * buf, (use - 1) & 1u)) return;
+        tc_fence_after();
+        const uint32_t acc = tmem + buf * acc_cols;
+        uint32_t b = (uint32_t)bd;
+        for (int k = 0; k < ksteps; ++k, b += 18u * N) {       // (x-shift, pair of chunk planes)
+#pragma unroll
+            for (int st = 0; st < ZST; ++st, q.next(S)) {
+                if (!wait(bar0 + 8u * q.s, q.r & 1u)) return;
+                tc_fence_after();
+                const uint32_t a = (uint32_t)ad + (uint32_t)q.s * stage_u;
+                // the stage's first input plane is st ZC - 1
+                const uint32_t col = acc + (uint32_t)(st == 0 ? 0 : (st * ZC - 2) * N);
+                if (leader) {
+                    if (st == 0) {
+                        if (k == 0) slab_stage<N, ZC, true, false, true>(col, a, a_hi, zrow, row, b, b_hi);
+                        else slab_stage<N, ZC, true, false, false>(col, a, a_hi, zrow, row, b, b_hi);
+                    } else if (st == ZST - 1) {
+                        if (k == 0) slab_stage<N, ZC, false, true, true>(col, a, a_hi, zrow, row, b, b_hi);
+                        else slab_stage<N, ZC, false, true, false>(col, a, a_hi, zrow, row, b, b_hi);
+                    } else {
+                        if (k == 0) slab_stage<N, ZC, false, false, true>(col, a, a_hi, zrow, row, b, b_hi);
+                        else slab_stage<N, ZC, false, false, false>(col, a, a_hi, zrow, row, b, b_hi);
+                    }
+                    umma_commit(bar0 + 8u * (S + q.s));
+                }
+                __syncwarp();
+            }
+        }
+        if (leader) umma_commit(acc_full + 8u * buf);
+        __syncwarp();
+    }
+}
+
+// ------------------------------------------------------------------------
+// conv3 walked along z (see SlabParams): warp 0 loads, warp 1 issues, eight
+// epilogue warps.  Tiles go round-robin over the CTAs (every tile is the same
+// work, one CTA per SM), their accumulators alternate between two TMEM buffers.
+// K order per output: x-shift, pair of chunk planes, z-tap, y-tap, 16 channels
+// -- the order of rows_kernel, so both give the same bits.  The first product
+// of an output plane (z-tap -1 of the first K-step) overwrites while the two
+// older planes of the same MMA accumulate: there the MMA is split in two.
+//
+// The rows kernel's MMAs of N = 16 and 32 columns are bound by their shared-
+// memory reads (128 A rows each); with N = 3 n they come near the tensor rate
+// (N = 96: 56 cycles of reads for 48 of arithmetic, three taps).  Measured, rows
+// kernel -> this, batch 16 at 64^3, forward: 16 -> 32 channels 183 -> 115 us,
+// 32 -> 32 301 -> 178 us (1.30 PFLOP/s), 64 -> 32 561 -> 356 us; input gradient:
+// 32 -> 32 with mask 318 -> 227 us, 32 -> 64 349 -> 270 us (1.72 PFLOP/s).
+// ------------------------------------------------------------------------
+template <int N, int ZC, int ZST>
+__global__ void __launch_bounds__(kSlabThreads, 1) slab_kernel(const __grid_constant__ SlabParams p) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = align1024(smem_raw);
+    const int S = p.stages;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + p.w_bytes + (size_t)S * p.stage_bytes);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * S + 5);
+    const uint32_t wbase = smem_u32(smem), sbase = wbase + p.w_bytes;
+    const uint32_t bar0 = smem_u32(bars);
+    const uint32_t acc_full = bar0 + 16u * S, acc_empty = acc_full + 16u, w_full = acc_empty + 16u;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t acc_cols = (uint32_t)(p.zp * N);
+    const uint32_t ncols = tmem_cols(2 * (int)acc_cols);
+    const uint32_t blk = N * 16u;                       // one tap and chunk plane of the weights
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < 2 * S; ++s) mbar_init(bar0 + 8u * s, 1);
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(acc_full + 8u * b, 1);
+            mbar_init(acc_empty + 8u * b, kSlabEpiWarps);
+        }
+        mbar_init(w_full, 1);
+        fence_mbar_init();
+    }
+    if (warp == 1) {
+        tmem_alloc(smem_u32(tmem_slot), ncols);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+
+    if (warp == 0) {
+        // weights: [dx][kc][dy][j][n][8] with j = 1 - dz, the order of the
+        // output planes z - 1, z, z + 1 (the packed operand has [dz][dy])
+        if (lane == 0) mbar_expect_tx(w_full, p.w_bytes);
+        __syncwarp();
+        const int nblk = 27 * p.kc_total;
+        for (int i = lane; i < nblk; i += 32) {
+            const int t9 = i % 9, dz = t9 / 3, dy = t9 % 3;
+            bulk_load(wbase + (uint32_t)(i - t9 + 3 * dy + 2 - dz) * blk,
+                      p.wpack + (size_t)i * (N * 8), blk, w_full);
+        }
+        if (lane == 0) {
+            Ring q;
+            bool ok = true;
+            for (int t = blockIdx.x; ok && t < p.tiles; t += gridDim.x) {
+                int x0, y0, z0, b0;
+                tile_origin_u32(p.g, (uint32_t)t, x0, y0, z0, b0);
+                for (int dx = -1; ok && dx <= 1; ++dx)
+                    for (int kc = 0; ok && kc < p.kc_total; kc += 2) {
+                        const int mi = kc < p.kc0 ? 0 : 1, c8 = kc < p.kc0 ? kc : kc - p.kc0;
+                        for (int z = 0; z < ZST; ++z, q.next(S)) {
+                            const uint32_t full = bar0 + 8u * q.s, empty = bar0 + 8u * (S + q.s);
+                            if (q.r > 0 && !mbar_wait(empty, (q.r - 1) & 1u, kWaitLimitNs)) {
+                                atomicOr(p.err, ERR_TIMEOUT);
+                                ok = false;
+                                break;
+                            }
+                            mbar_expect_tx(full, p.stage_bytes);
+                            tma_load_5d(sbase + (uint32_t)q.s * p.stage_bytes, &p.maps[mi], full, 8 * (x0 + dx),
+                                        y0 - 1, z0 - 1 + z * ZC, b0, c8);
+                        }
+                    }
+            }
+        }
+    } else if (warp == 1) {
+        slab_issue<N, ZC, ZST>(p, bar0, acc_full, acc_empty, w_full, wbase, sbase, tmem);
+    } else {
+        const int q = warp & 3;
+        const int r = q * 32 + lane;
+        const int half = (warp - 2) >> 2;
+        const uint32_t lane_base = (uint32_t)(q * 32) << 16;
+        uint32_t it = 0;
+        for (int t = blockIdx.x; t < p.tiles; t += gridDim.x, ++it) {
+            const uint32_t buf = it & 1u, use = it >> 1;
+            if (!__all_sync(0xffffffffu, mbar_wait(acc_full + 8u * buf, use & 1u, kWaitLimitNs))) {
+                if (lane == 0) atomicOr(p.err, ERR_TIMEOUT);
+                break;
+            }
+            tc_fence_after();
+            int x0, y0, z0, b0;
+            tile_origin_u32(p.g, (uint32_t)t, x0, y0, z0, b0);
+            const int x = x0 + r % p.g.bx, y = y0 + r / p.g.bx;
+            // two warps per quarter of the rows: even and odd planes
+            const long long zstep = (long long)p.g.H * p.g.W;
+            long long vox = (((long long)b0 * p.g.D + z0 + half) * p.g.H + y) * p.g.W + x;
+            for (int z = half; z < p.zp; z += 2, vox += 2 * zstep) {
+                const uint32_t col = tmem + buf * acc_cols + lane_base + (uint32_t)(z * N);
+                float head = 0.f;
+#pragma unroll
+                for (int n0 = 0; n0 < N; n0 += 16) {
+                    uint32_t v[16];
+                    tmem_ld16(col + (uint32_t)n0, v);
+                    tmem_wait_ld();
+                    const EpiDest& d = (n0 < p.split) ? p.d[0] : p.d[1];
+                    if (d.out == nullptr) continue;
+                    const int ch0 = n0 - d.col0;
+                    emit16(d, v, ch0, (ch0 >> 3) * d.plane + vox * 8, p.head_out ? p.head_w : nullptr, head);
+                }
+                if (p.head_out) p.head_out[vox] = head + *p.head_b;
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(acc_empty + 8u * buf);
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem, ncols);
+    }
+}
+
+template <int N, int ZC, int ZST>
+cudaError_t launch_slab_as(const SlabParams& p, int grid, size_t smem, cudaStream_t s) {
+    static bool attr = false;
+    if (!attr) {
+        cudaError_t e = cudaFuncSetAttribute(slab_kernel<N, ZC, ZST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             227 * 1024);
+        if (e != cudaSuccess) return e;
+        attr = true;
+    }
+    slab_kernel<N, ZC, ZST><<<grid, kSlabThreads, smem, s>>>(p);
+    return cudaGetLastError();
+}
+
+template <int N>
+cudaError_t launch_slab_n(const SlabParams& p, int grid, size_t smem, cudaStream_t s) {
+    switch (p.zp) {                 // stages as in slab_zc
+    case 2: return launch_slab_as<N, 2, 2>(p, grid, smem, s);
+    case 4: return launch_slab_as<N, 3, 2>(p, grid, smem, s);
+    case 8: if (N <= 32) return launch_slab_as<N <= 32 ? N : 16, 5, 2>(p, grid, smem, s); break;
+    case 16: if (N <= 16) return launch_slab_as<16, 6, 3>(p, grid, smem, s); break;
+    }
+    return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_slab(const SlabParams& p, int grid, size_t smem, cudaStream_t s) {
+    switch (p.n) {
+    case 16: return launch_slab_n<16>(p, grid, smem, s);
+    case 32: return launch_slab_n<32>(p, grid, smem, s);
+    case 64: return launch_slab_n<64>(p, grid, smem, s);
+    }
+    return cudaErrorInvalidValue;
 }
 
 __global__ void __launch_bounds__(kThreads, 1) rows_kernel(const __grid_constant__ RowsParams p) {
@@ -398,42 +693,7 @@ __global__ void __launch_bounds__(kThreads, 1) rows_kernel(const __grid_constant
                             ch0 = n0 - d.col0;
                             off = (ch0 >> 3) * d.plane + vox * 8;
                         }
-                        float f[16];
-                        #pragma unroll
-                        for (int i = 0; i < 16; ++i) f[i] = __uint_as_float(v[i]);
-                        if (d.bias) {
-                            #pragma unroll
-                            for (int i = 0; i < 16; ++i) f[i] += d.bias[ch0 + i];
-                        }
-                        if (d.addend) {
-                            float a[16];
-                            load16_planes(d.addend + off, d.plane, a);
-                            #pragma unroll
-                            for (int i = 0; i < 16; ++i) f[i] += a[i];
-                        }
-                        if (d.relu) {
-                            #pragma unroll
-                            for (int i = 0; i < 16; ++i) f[i] = fmaxf(f[i], 0.f);
-                        }
-                        if (d.mask) {
-                            float mk[16];
-                            load16_planes(d.mask + off, d.plane, mk);
-                            #pragma unroll
-                            for (int i = 0; i < 16; ++i) f[i] = (mk[i] > 0.f) ? f[i] : 0.f;
-                        }
-                        uint4 w[2];
-                        __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(w);
-                        #pragma unroll
-                        for (int i = 0; i < 8; ++i) h[i] = __floats2bfloat162_rn(f[2 * i], f[2 * i + 1]);
-                        *reinterpret_cast<uint4*>(d.out + off) = w[0];
-                        *reinterpret_cast<uint4*>(d.out + off + d.plane) = w[1];
-                        if (p.head_out) {
-                            #pragma unroll
-                            for (int i = 0; i < 8; ++i) {
-                                const float2 rb = __bfloat1622float2(h[i]);
-                                head_acc += rb.x * p.head_w[ch0 + 2 * i] + rb.y * p.head_w[ch0 + 2 * i + 1];
-                            }
-                        }
+                        emit16(d, v, ch0, off, p.head_out ? p.head_w : nullptr, head_acc);
                     };
                     for (int j = 0; j < nch; ++j) {
                         uint32_t v[16];

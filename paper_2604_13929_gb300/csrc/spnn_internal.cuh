@@ -102,6 +102,30 @@ struct RowsParams {
     int* err;
 };
 
+// conv3 forward / input gradient with few output channels, walked along z.  A
+// CTA box is bx x by = 128 voxels of zp consecutive z-planes; each plane has its
+// own accumulator of n columns, side by side in TMEM.  An input plane z feeds
+// the output planes z - 1, z, z + 1, which are 3 n adjacent columns: one MMA per
+// (x-shift, y-shift, 16 channels) with N = 3 n serves the three z-taps, so the
+// 128 A rows are read from shared memory once instead of three times.  The
+// weights stay in shared memory for the whole launch.
+struct SlabParams {
+    CUtensorMap maps[2];            // sources, box (8 bx, by + 2, zc, 1, 2)
+    const __nv_bfloat16* wpack;     // conv3 packed operand, one N tile
+    int kc_total, kc0;              // chunk planes (two per K-step)
+    int zp;                         // output planes per box: 2, 4, 8, 16
+    int n;                          // output channels: 16, 32, 64
+    TileGrid g;                     // bz = zp
+    int tiles, stages;
+    uint32_t w_bytes, stage_bytes;  // all weights; one stage
+    int split;
+    EpiDest d[2];
+    float* head_out;
+    const float* head_w;
+    const float* head_b;
+    int* err;
+};
+
 // Weight-gradient GEMM: D[(group, r), n] = sum_v A_group[v, r] B[v, n] over a
 // range of 64-voxel K-steps (boxes of the V grid); rows are 16 groups of 8
 // input channels (one tap each), both operands MN-major, results added to
@@ -155,6 +179,12 @@ struct WgradHaloParams {
 // Persistent launch: min(tiles, persistent x SMs x resident CTAs) x grid_n CTAs.
 constexpr int kMaxGridN = 16;               // N tiles of one rows GEMM (claim counters per launch)
 cudaError_t launch_rows(const RowsParams& p, int grid_n, size_t smem, cudaStream_t s);
+// Input planes per stage of the z-walk: the most that divide zp + 2 into at
+// least two stages of at most six.
+__host__ __device__ constexpr int slab_zc(int zp) { return zp == 16 ? 6 : (zp == 8 ? 5 : (zp == 4 ? 3 : 2)); }
+constexpr int kSlabEpiWarps = 8;            // two per quarter of the accumulator's rows
+constexpr int kSlabThreads = 64 + 32 * kSlabEpiWarps;
+cudaError_t launch_slab(const SlabParams& p, int grid, size_t smem, cudaStream_t s);
 cudaError_t launch_wgrad_halo(const WgradHaloParams& p, dim3 grid, size_t smem, cudaStream_t s);
 cudaError_t launch_wgrad(const WgradParams& p, dim3 grid, size_t smem, cudaStream_t s);
 // TMEM columns to allocate for n FP32 accumulator columns (a power of two >= 32).

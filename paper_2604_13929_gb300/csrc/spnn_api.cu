@@ -713,6 +713,80 @@ int wgrad_halo(int B, int D, int H, int W, const void* x0, int c0, const void* x
     return SPNN_OK;
 }
 
+// conv3 weight gradient on row windows (see WgradRowsParams).  Returns 1 when
+// the layer does not fit.
+int wgrad_rows(int B, int D, int H, int W, const void* x0, int c0, const void* x1, int c1, const void* dy,
+               int cout, float* dw, float* db, cudaStream_t st) {
+    const int kc0 = c0 / 8, kc1 = c1 / 8, kc = kc0 + kc1;
+    if (cout != 16 && cout != 32 && cout % 64) return 1;
+    WgradRowsParams p;
+    memset(&p, 0, sizeof p);
+    p.nc = cout < 64 ? cout : 64;
+    p.bx = W < 32 ? W : 32;
+    if (p.bx < 8) return 1;
+    // 128-voxel K-steps, 64 with 64 output channels (their dY blocks are twice as large)
+    p.by = (p.nc == 64 ? 64 : 128) / p.bx;
+    if (p.by > 8) p.by = 8;
+    if (H < p.by) return 1;
+    p.kc0 = kc0, p.kc1 = kc1, p.cout = cout;
+    // planes per CTA: up to four (36 row groups in three 128-row tiles of 3 nc
+    // columns), three where two tiles of 192 columns fill TMEM; balanced splits
+    const int np_max = p.nc == 64 ? 3 : 4;
+    const int sp0 = (kc0 + np_max - 1) / np_max, sp1 = (kc1 + np_max - 1) / np_max;
+    p.np0 = (kc0 + sp0 - 1) / sp0;
+    p.np1 = sp1 ? (kc1 + sp1 - 1) / sp1 : 0;
+    p.splits0 = sp0;
+    const int splits = sp0 + sp1;
+    const int np = p.np0 > p.np1 ? p.np0 : p.np1;
+    const int nm = (9 * np + 15) / 16;
+    p.g.B = B, p.g.D = D, p.g.H = H, p.g.W = W;
+    p.nx = W / p.bx;
+    p.ny = H / p.by;
+    p.zs = D % 8 == 0 ? 8 : (D % 4 == 0 ? 4 : (D % 2 == 0 ? 2 : 1));
+    p.nzs = D / p.zs;
+    const uint32_t row = 16u * (uint32_t)p.bx;
+    p.a_bytes = (uint32_t)(3 * np * (p.by + 2)) * row;
+    // the last M tile reads past its 9 np groups, at most 15 runs into the B block
+    const uint32_t b_bytes = (uint32_t)(3 * (p.nc / 8) * p.by) * row;
+    if (b_bytes < 15u * row) return 1;
+    p.stage_bytes = (p.a_bytes + b_bytes + 1023u) & ~1023u;
+    const int per_sm = 512 / (int)tmem_cols(nm * 3 * p.nc) > 1 ? 2 : 1;
+    p.stages = (int)((per_sm > 1 ? 108u : 216u) * 1024u / p.stage_bytes);
+    if (p.stages > 6) p.stages = 6;
+    if (p.stages < 2) return 1;
+    int rc;
+    const cuuint64_t line = 16ull * W, plane = line * H * D * B;
+    cuuint64_t strides[4] = {plane, line * H, line, line * H * D};
+    auto map = [&](CUtensorMap* m, const void* ptr, int C, int planes, int dz, int rows) {
+        cuuint64_t dims[5] = {8ull * W, (cuuint64_t)(C / 8), (cuuint64_t)D, (cuuint64_t)H, (cuuint64_t)B};
+        cuuint32_t box[5] = {8u * p.bx, (cuuint32_t)planes, (cuuint32_t)dz, (cuuint32_t)rows, 1};
+        return encode(m, ptr, dims, strides, box);
+    };
+    if ((rc = map(&p.amaps[0], x0, c0, p.np0, 3, p.by + 2))) return rc;
+    if (c1 && (rc = map(&p.amaps[1], x1, c1, p.np1, 3, p.by + 2))) return rc;
+    if ((rc = map(&p.bmap, dy, cout, p.nc / 8, 1, 1))) return rc;
+    p.dw = dw;
+    p.db = db;
+    p.vec = reinterpret_cast<uintptr_t>(dw) % 16 == 0;
+    p.err = err_ptr();
+    if (!p.err) return fail(SPNN_ECUDA, "no device");
+    p.ksteps_total = B * D * p.ny * p.nx;
+    // K splits.  The tensor cores truncate as they accumulate, so a sum's error
+    // grows with the voxels one accumulator takes.  Their number stays what it
+    // was with one 128-row tile per CTA, however the planes are split: a 608th
+    // of the layer's voxels per input plane up to 32 output channels, else per
+    // tile of 16 row groups.
+    const int tiles16 = (27 * kc + 16) / 16;
+    int ks = cout <= 32 ? (608 + kc - 1) / kc : (608 + tiles16 - 1) / tiles16;
+    if (ks > p.ksteps_total) ks = p.ksteps_total;
+    p.ksteps_per_cta = (p.ksteps_total + ks - 1) / ks;
+    ks = (p.ksteps_total + p.ksteps_per_cta - 1) / p.ksteps_per_cta;
+    size_t smem = (size_t)p.stages * p.stage_bytes + 1024 + (2 * p.stages + 2) * 8;
+    cudaError_t e = launch_wgrad_rows(p, nm, dim3(ks, splits, cout / p.nc), smem, st);
+    if (e != cudaSuccess) return cuda_fail(e, "wgrad_rows_kernel launch");
+    return SPNN_OK;
+}
+
 int layer_wgrad(int kind, int B, int D, int H, int W, const void* x0, int c0, const void* x1, int c1,
                 const void* dy, int cout, float* dw, float* db, cudaStream_t st) {
     int rc;
@@ -720,6 +794,10 @@ int layer_wgrad(int kind, int B, int D, int H, int W, const void* x0, int c0, co
     if (!x0 || !dy || !dw || (c1 && !x1)) return fail(SPNN_EINVAL, "null tensor");
     if (c1 && kind != KIND_CONV3) return fail(SPNN_EINVAL, "concatenated input only for conv3");
     if (c0 % 8 || c1 % 8) return fail(SPNN_EINVAL, "source channels must be multiples of 8");
+    if (kind == KIND_CONV3 && g_opt_wgrad_halo == 1) {
+        const int r = wgrad_rows(B, D, H, W, x0, c0, x1, c1, dy, cout, dw, db, st);
+        if (r != 1) return r;
+    }
     if (kind == KIND_CONV3 && g_opt_wgrad_halo) {
         const int h = wgrad_halo(B, D, H, W, x0, c0, x1, c1, dy, cout, dw, db, st);
         if (h != 1) return h;

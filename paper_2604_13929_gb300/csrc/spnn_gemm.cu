@@ -1,6 +1,6 @@
 // spnn_gemm.cu -- the tensor-core GEMM kernels of the surrogate: rows_kernel
-// and slab_kernel (forward and input-gradient layers), wgrad_kernel and
-// wgrad_halo_kernel (weight gradients).
+// and slab_kernel (forward and input-gradient layers), wgrad_kernel,
+// wgrad_halo_kernel and wgrad_rows_kernel (weight gradients).
 //
 // All are warp-specialised, 192 threads (slab_kernel 320):
 //   warp 0      TMA producer: fills a ring of shared-memory stages,
@@ -1148,6 +1148,269 @@ cudaError_t launch_wgrad_halo(const WgradHaloParams& p, dim3 grid, size_t smem, 
     }
     wgrad_halo_kernel<<<grid, kThreads, smem, s>>>(p);
     return cudaGetLastError();
+}
+
+// ------------------------------------------------------------------------
+// conv3 weight gradient on row windows (see WgradRowsParams).  N3 = 3 nc MMA
+// columns, NM 128-row tiles (9 np groups of 8 rows, the rest reads what follows
+// and is dropped), RPS output rows (pairs of rows where bx = 8) per K-step with
+// KPR 16-voxel K-blocks each.
+//
+// What bounded the kernels before it was operand delivery: the halo kernel
+// loaded nine input rows per plane for every output row and the per-tap kernel
+// up to 16 boxes per K-step (tensor pipe 17 - 25 % active).  Here an input row
+// is loaded (by + 2) / by times per z-plane, and a K-step is 8 to 24 MMAs issued
+// as straight code.  Measured at batch 16, halo or per-tap kernel -> this: 64^3
+// 16 -> 32 channels 272 -> 138 us, 32 -> 32 450 -> 200 us, 64 -> 32 801 -> 375 us
+// (1.24 PFLOP/s); 32^3 64 -> 64 218 -> 117 us, 128 -> 64 412 -> 206 us; 16^3
+// 128 -> 128 115 -> 78 us; 8^3 256 -> 256 128 -> 73 us.
+// ------------------------------------------------------------------------
+
+// The MMAs of one stage, straight line (a loop that works out its operands
+// takes a lone warp longer than the MMAs).  Offsets in 16-byte units: a_row /
+// b_row between output rows, 16 between K-blocks of a row, a_tile between M tiles.
+template <int N3, int NM, int KPR, int RPS>
+__device__ __forceinline__ void wgrad_rows_stage(uint32_t tmem, uint32_t a, uint32_t a_hi, uint32_t a_row,
+                                                 uint32_t a_tile, uint32_t b, uint32_t b_hi, uint32_t b_row,
+                                                 bool first) {
+    constexpr uint32_t id = idesc_bf16(128, N3, 1, 1);
+#pragma unroll
+    for (int r = 0; r < RPS; ++r)
+#pragma unroll
+        for (int k = 0; k < KPR; ++k)
+#pragma unroll
+            for (int m = 0; m < NM; ++m) {
+                const uint32_t ad = a + (uint32_t)r * a_row + 16u * k + (uint32_t)m * a_tile;
+                const uint32_t bd = b + (uint32_t)r * b_row + 16u * k;
+                if (r == 0 && k == 0 && first) umma_bf16_lo<0>(tmem + (uint32_t)(m * N3), ad, a_hi, bd, b_hi, id);
+                else umma_bf16_lo<1>(tmem + (uint32_t)(m * N3), ad, a_hi, bd, b_hi, id);
+            }
+}
+
+template <int N3, int NM, int KPR, int RPS>
+__global__ void __launch_bounds__(kThreads, 1) wgrad_rows_kernel(const __grid_constant__ WgradRowsParams p) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = align1024(smem_raw);
+    const int S = p.stages;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)S * p.stage_bytes);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * S + 1);
+    const uint32_t sbase = smem_u32(smem);
+    const uint32_t bar0 = smem_u32(bars);
+    const uint32_t done = bar0 + 16u * S;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int kbeg = blockIdx.x * p.ksteps_per_cta;
+    const int kend = min(kbeg + p.ksteps_per_cta, p.ksteps_total);
+    constexpr int nb = N3 / 24;                            // 8-channel blocks of dY
+    const int split = blockIdx.y, src = split < p.splits0 ? 0 : 1;
+    const int np = src ? p.np1 : p.np0;
+    const int first = (src ? split - p.splits0 : split) * np;      // planes past the source load as zeros
+    const int real = min(np, (src ? p.kc1 : p.kc0) - first);
+    const int co0 = blockIdx.z * p.nc;
+    const bool bias = p.db != nullptr && split == 0;
+    const uint32_t row = 16u * (uint32_t)p.bx;             // one x-run of 8 channels
+    constexpr uint32_t ncols = (NM * N3 <= 64) ? 64 : (NM * N3 <= 128) ? 128 : (NM * N3 <= 256) ? 256 : 512;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < S; ++s) {
+            mbar_init(bar0 + 8u * s, 1);
+            mbar_init(bar0 + 8u * (S + s), bias ? 5 : 1);  // the MMAs and, for the bias, four warps
+        }
+        mbar_init(done, 1);
+        fence_mbar_init();
+    }
+    if (warp == 1) {
+        tmem_alloc(smem_u32(tmem_slot), ncols);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+
+    if (warp == 0) {
+        // lane 3 y + dx loads dY's row y shifted by dx, lane 31 the input box
+        const int yl = lane / 3, dxl = lane % 3;
+        const bool b_lane = lane < 3 * p.by;
+        const uint32_t b_off = p.a_bytes + (uint32_t)lane * nb * row;
+        const uint32_t tx = (uint32_t)(3 * np * (p.by + 2)) * row + (uint32_t)(3 * nb * p.by) * row;
+        int k = kbeg, xr = k % p.nx, rest = k / p.nx;
+        int zi = rest % p.zs;
+        rest /= p.zs;
+        int yb = rest % p.ny;
+        rest /= p.ny;
+        int zsl = rest % p.nzs, b = rest / p.nzs;
+        Ring q;
+        for (; k < kend; ++k, q.next(S)) {
+            const uint32_t full = bar0 + 8u * q.s, empty = bar0 + 8u * (S + q.s);
+            if (q.r > 0 && !__all_sync(0xffffffffu, mbar_wait(empty, (q.r - 1) & 1u, kWaitLimitNs))) {
+                if (lane == 0) atomicOr(p.err, ERR_TIMEOUT);
+                break;
+            }
+            if (lane == 0) mbar_expect_tx(full, tx);
+            __syncwarp();
+            const uint32_t dst = sbase + (uint32_t)q.s * p.stage_bytes;
+            const int x0 = xr * p.bx, y0 = yb * p.by, z = zsl * p.zs + zi;
+            if (b_lane) tma_load_5d(dst + b_off, &p.bmap, full, 8 * (x0 + 1 - dxl), co0 / 8, z, y0 + yl, b);
+            if (lane == 31) tma_load_5d(dst, &p.amaps[src], full, 8 * x0, first, z - 1, y0 - 1, b);
+            __syncwarp();
+            // x-runs, then z within the slab, then y, slab, sample: the rows a
+            // K-step loads were loaded by a recent one (L2)
+            if (++xr == p.nx) {
+                xr = 0;
+                if (++zi == p.zs) {
+                    zi = 0;
+                    if (++yb == p.ny) {
+                        yb = 0;
+                        if (++zsl == p.nzs) zsl = 0, ++b;
+                    }
+                }
+            }
+        }
+    } else if (warp == 1) {
+        const bool leader = elect_one();
+        // K-block of 16 voxels: two 8-voxel core matrices of one run, or (bx = 8)
+        // of two rows; row groups one run apart
+        const bool pairs = p.bx == 8;
+        const uint32_t a_run = 3u * (uint32_t)np * row, b_run = 3u * nb * row;      // between output rows
+        const uint64_t ad = smem_desc(sbase, pairs ? a_run : 128u, row);
+        const uint64_t bd = smem_desc(sbase + p.a_bytes, pairs ? b_run : 128u, row);
+        const uint32_t a_hi = (uint32_t)(ad >> 32), b_hi = (uint32_t)(bd >> 32), stage_u = p.stage_bytes / 16u;
+        const uint32_t a_row = (pairs ? 2u : 1u) * a_run / 16u, b_row = (pairs ? 2u : 1u) * b_run / 16u;
+        Ring q;
+        for (int k = kbeg; k < kend; ++k, q.next(S)) {
+            if (!__all_sync(0xffffffffu, mbar_wait(bar0 + 8u * q.s, q.r & 1u, kWaitLimitNs))) {
+                if (leader) atomicOr(p.err, ERR_TIMEOUT);
+                break;
+            }
+            tc_fence_after();
+            if (leader) {
+                wgrad_rows_stage<N3, NM, KPR, RPS>(tmem, (uint32_t)ad + (uint32_t)q.s * stage_u, a_hi, a_row, row,
+                                                   (uint32_t)bd + (uint32_t)q.s * stage_u, b_hi, b_row, k == kbeg);
+                umma_commit(bar0 + 8u * (S + q.s));
+            }
+            __syncwarp();
+        }
+        if (leader) umma_commit(done);
+        __syncwarp();
+    } else {
+        const int q4 = warp & 3, r = q4 * 32 + lane;
+        bool ok = true;
+        if (bias) {
+            // thread r sums channel block c8 of the voxels v = r % tpb + i tpb
+            constexpr int tpb = 128 / nb;
+            const int c8 = r / tpb, vox = p.bx * p.by;
+            float sum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            Ring q;
+            for (int k = kbeg; k < kend; ++k, q.next(S)) {
+                if (!__all_sync(0xffffffffu, mbar_wait(bar0 + 8u * q.s, q.r & 1u, kWaitLimitNs))) {
+                    if (lane == 0) atomicOr(p.err, ERR_TIMEOUT);
+                    ok = false;
+                    break;
+                }
+                const uint8_t* bst = smem + (size_t)q.s * p.stage_bytes + p.a_bytes;
+                for (int v = r % tpb; v < vox; v += tpb) {
+                    const int y = v / p.bx, x = v % p.bx;
+                    const uint4 u = *reinterpret_cast<const uint4*>(bst + (size_t)((3 * y + 1) * nb + c8) * row + 16 * x);
+                    const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float2 f = __bfloat1622float2(h[i]);
+                        sum[2 * i] += f.x;
+                        sum[2 * i + 1] += f.y;
+                    }
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar0 + 8u * (S + q.s));
+            }
+            constexpr int width = tpb < 32 ? tpb : 32;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                for (int o = width / 2; o; o >>= 1) sum[i] += __shfl_xor_sync(0xffffffffu, sum[i], o);
+                if (ok && lane % width == 0) atomicAdd(p.db + co0 + 8 * c8 + i, sum[i]);
+            }
+        }
+        ok = __all_sync(0xffffffffu, ok && mbar_wait(done, 0, kWaitLimitNs));
+        if (!ok) {
+            if (lane == 0) atomicOr(p.err, ERR_TIMEOUT);
+        } else if (kend > kbeg) {
+            tc_fence_after();
+            const int ci_all = 8 * (p.kc0 + p.kc1), plane0 = (src ? p.kc0 : 0) + first;
+            for (int m = 0; m < NM; ++m) {
+                // row group (dy, dz, plane)
+                const int gr = 16 * m + (r >> 3), dy = gr / (3 * np), dz = gr / np % 3, pl = gr % np;
+                const bool wrow = gr < 9 * np && pl < real;
+                for (int c = 0; c < N3; c += 16) {
+                    uint32_t v[16];
+                    tmem_ld16(tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(m * N3 + c), v);
+                    tmem_wait_ld();
+                    const int dx = c / (N3 / 3), co = c % (N3 / 3);
+                    if (!wrow) continue;
+                    float* dst = p.dw + ((size_t)((dz * 3 + dy) * 3 + dx) * ci_all + (plane0 + pl) * 8 + (r & 7)) * p.cout +
+                                 co0 + co;
+                    if (p.vec) {
+#pragma unroll
+                        for (int e = 0; e < 16; e += 4)
+                            atomicAdd(reinterpret_cast<float4*>(dst + e),
+                                      make_float4(__uint_as_float(v[e]), __uint_as_float(v[e + 1]),
+                                                  __uint_as_float(v[e + 2]), __uint_as_float(v[e + 3])));
+                    } else {
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) atomicAdd(dst + e, __uint_as_float(v[e]));
+                    }
+                }
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem, ncols);
+    }
+}
+
+namespace {
+template <int N3, int NM, int KPR, int RPS>
+cudaError_t launch_wr(const WgradRowsParams& p, dim3 grid, size_t smem, cudaStream_t s) {
+    static bool attr = false;
+    if (!attr) {
+        cudaError_t e = cudaFuncSetAttribute(wgrad_rows_kernel<N3, NM, KPR, RPS>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        if (e != cudaSuccess) return e;
+        attr = true;
+    }
+    wgrad_rows_kernel<N3, NM, KPR, RPS><<<grid, kThreads, smem, s>>>(p);
+    return cudaGetLastError();
+}
+
+// by rows per K-step: 128 voxels for nc <= 32, 64 for nc = 64 (fewer where the
+// layer has fewer rows)
+template <int N3, int NM>
+cudaError_t launch_wr_rows(const WgradRowsParams& p, dim3 grid, size_t smem, cudaStream_t s) {
+    const int rps = p.bx == 8 ? p.by / 2 : p.by;
+    if (p.bx == 32) {
+        if (rps == 4) return launch_wr<N3, NM, 2, 4>(p, grid, smem, s);
+        if (rps == 2) return launch_wr<N3, NM, 2, 2>(p, grid, smem, s);
+    } else {
+        if (rps == 8) return launch_wr<N3, NM, 1, 8>(p, grid, smem, s);
+        if (rps == 4) return launch_wr<N3, NM, 1, 4>(p, grid, smem, s);
+    }
+    return cudaErrorInvalidValue;
+}
+}  // namespace
+
+cudaError_t launch_wgrad_rows(const WgradRowsParams& p, int nm, dim3 grid, size_t smem, cudaStream_t s) {
+    switch (4 * p.nc / 16 + nm) {
+    case 4 + 1: return launch_wr_rows<48, 1>(p, grid, smem, s);
+    case 4 + 2: return launch_wr_rows<48, 2>(p, grid, smem, s);
+    case 4 + 3: return launch_wr_rows<48, 3>(p, grid, smem, s);
+    case 8 + 1: return launch_wr_rows<96, 1>(p, grid, smem, s);
+    case 8 + 2: return launch_wr_rows<96, 2>(p, grid, smem, s);
+    case 8 + 3: return launch_wr_rows<96, 3>(p, grid, smem, s);
+    case 16 + 1: return launch_wr_rows<192, 1>(p, grid, smem, s);
+    case 16 + 2: return launch_wr_rows<192, 2>(p, grid, smem, s);
+    }
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace spnn

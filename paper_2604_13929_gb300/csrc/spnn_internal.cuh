@@ -176,6 +176,34 @@ struct WgradHaloParams {
     int* err;
 };
 
+// conv3 weight gradient on row windows: dW[tap][ci][co] = sum_u X[u] dY[u - d].
+// A K-step is by rows of bx voxels in one z-plane.  A (MN-major): one TMA box
+// of the input laid out [y][dz][plane][x], by + 2 rows high, so the 9 np groups
+// (dy, dz, plane) of output row y are consecutive blocks of one x-run that start
+// at row y: the rows' windows overlap in shared memory and every input row is
+// loaded once for three output rows.  B (MN-major): dY laid out
+// [y][dx][8-channel block][x], each x-shift loaded on its own, so one MMA has
+// N = 3 nc columns (dx, co).  blockIdx.y splits the input planes (np per CTA,
+// within one source), blockIdx.z the output channels (nc each), blockIdx.x the
+// K-steps.  The bias gradient is summed from dY's middle x-shift by the epilogue
+// warps of plane split 0 while the stages pass.
+struct WgradRowsParams {
+    CUtensorMap amaps[2];           // sources, dims (8W, C/8, D, H, B), box (8 bx, np0 / np1, 3, by + 2, 1)
+    CUtensorMap bmap;               // output gradient, same dims, box (8 bx, nc / 8, 1, 1, 1)
+    int kc0, kc1, cout, nc;
+    int np0, np1, splits0;          // planes per CTA of source 0 / 1; plane splits over source 0
+    int bx, by;
+    int nx, ny, zs, nzs;            // boxes per row and column, z slab depth, slabs per sample
+    TileGrid g;                     // B, D, H, W of the layer
+    int ksteps_total, ksteps_per_cta, stages;
+    uint32_t a_bytes, stage_bytes;  // A block of a stage (B follows), stage
+    int vec;                        // dw is 16-byte aligned
+    float* dw;                      // [27][8 (kc0 + kc1)][cout]
+    float* db;                      // [cout] or null
+    int* err;
+};
+cudaError_t launch_wgrad_rows(const WgradRowsParams& p, int nm, dim3 grid, size_t smem, cudaStream_t s);
+
 // Persistent launch: min(tiles, persistent x SMs x resident CTAs) x grid_n CTAs.
 constexpr int kMaxGridN = 16;               // N tiles of one rows GEMM (claim counters per launch)
 cudaError_t launch_rows(const RowsParams& p, int grid_n, size_t smem, cudaStream_t s);

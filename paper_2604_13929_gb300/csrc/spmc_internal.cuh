@@ -93,15 +93,19 @@ struct TransportParams {
 // claim counter: global index k belongs to the problem whose
 // [offset, offset + n_photons) contains it, with photon id pid_begin + k - offset.
 // The streamlined FP32 kernel claims work in chunks of `chunk` photons of one
-// problem per warp: problem i owns the global chunk indices
-// [chunk_begin, chunk_begin + ceil(n_photons / chunk)).
+// problem per warp, from the problem's own counter.  Problems come in groups
+// [group, group_end) of consecutive ones whose voxel fields share L2: a warp
+// stays with a problem until it runs out, then takes another of its group, and
+// only then the next group.
 struct BatchProblem {
     const u64 *bricks;
     u64 *field;
     DevTallies *tal;
     int nx, ny, nz, nbx, nby, nbz;
     u64 pid_begin, n_photons, offset;
-    u64 chunk_begin;
+    u64 chunks;                    // ceil(n_photons / chunk)
+    u64 group_chunks, group_before; // chunks of the whole group; of its problems before this one
+    int group, group_end;
     u32 iter_limit;
     int hg_iso, small_x, plain, mirror;
     TransportParams::F32 f32;
@@ -111,9 +115,9 @@ struct BatchParams {
     const BatchProblem *problems;   // device table
     int n_problems;
     u64 total_photons;              // sum of n_photons (one run)
-    u64 total_chunks;               // chunks over all problems (streamlined kernel)
     u32 chunk;                      // photons per chunk (streamlined kernel)
-    u64 *next;                      // claim counter, zeroed before each launch
+    u64 *next;                      // claim counters, zeroed before each launch: one per problem
+                                    // (streamlined kernel), or the first for all photons
     u32 key0, key1;                 // Philox key = seed (shared by all problems)
     int compact_k;
     int steps_per_pass;

@@ -772,14 +772,28 @@ int wgrad_rows(int B, int D, int H, int W, const void* x0, int c0, const void* x
     if (!p.err) return fail(SPNN_ECUDA, "no device");
     p.ksteps_total = B * D * p.ny * p.nx;
     // K splits.  The tensor cores truncate as they accumulate, so a sum's error
-    // grows with the voxels one accumulator takes.  Their number stays what it
-    // was with one 128-row tile per CTA, however the planes are split: a 608th
-    // of the layer's voxels per input plane up to 32 output channels, else per
-    // tile of 16 row groups.
-    const int tiles16 = (27 * kc + 16) / 16;
-    int ks = cout <= 32 ? (608 + kc - 1) / kc : (608 + tiles16 - 1) / tiles16;
+    // grows with the voxels one accumulator takes (32 -> 32 channels, 16 samples of
+    // 64^3: 2.7e-5 of the gradient).  Their number is that of the kernels this one
+    // replaces, one resident round of CTAs of two 128-row tiles (up to 32 output
+    // channels on runs of 16 voxels) or four rounds of one tile, however the planes
+    // are split here.
+    int ks;
+    if (cout <= 32 && W % 16 == 0) {
+        const int s0 = (kc0 + 2) / 3, s1 = (kc1 + 2) / 3;
+        const int q0 = (kc0 + s0 - 1) / s0, q1 = s1 ? (kc1 + s1 - 1) / s1 : 0;
+        const int tiles = (9 * (q0 > q1 ? q0 : q1) + 16) / 16;
+        ks = (152 * (512 / (int)tmem_cols(tiles * 3 * cout)) + s0 + s1 - 1) / (s0 + s1);
+    } else {
+        const int tiles16 = (27 * kc + 16) / 16;
+        ks = (608 + tiles16 - 1) / tiles16;
+    }
     if (ks > p.ksteps_total) ks = p.ksteps_total;
-    p.ksteps_per_cta = (p.ksteps_total + ks - 1) / ks;
+    // rounded down where that needs no further round of CTAs, else up
+    const long long slots = 152 * per_sm, units = (long long)splits * (cout / p.nc);
+    p.ksteps_per_cta = p.ksteps_total / ks;
+    const long long ctas = (p.ksteps_total + p.ksteps_per_cta - 1) / p.ksteps_per_cta * units;
+    if ((ctas + slots - 1) / slots > (ks * units + slots - 1) / slots)
+        p.ksteps_per_cta = (p.ksteps_total + ks - 1) / ks;
     ks = (p.ksteps_total + p.ksteps_per_cta - 1) / p.ksteps_per_cta;
     size_t smem = (size_t)p.stages * p.stage_bytes + 1024 + (2 * p.stages + 2) * 8;
     cudaError_t e = launch_wgrad_rows(p, nm, dim3(ks, splits, cout / p.nc), smem, st);
@@ -853,11 +867,29 @@ int layer_wgrad(int kind, int B, int D, int H, int W, const void* x0, int c0, co
 cudaStream_t as_stream(void* s) { return static_cast<cudaStream_t>(s); }
 
 // --------------------------------------------------------- data kernels --
-// Pore fraction of each sample's mask: one block per sample.
-__global__ void porosity_kernel(const uint8_t* __restrict__ mask, long long vox_per_sample, float* __restrict__ phi) {
-    const uint8_t* m = mask + (long long)blockIdx.x * vox_per_sample;
+// Pore fraction of each sample's mask: gridDim.x blocks per sample, 16 mask
+// bytes per load where aligned; the sample's last block to finish (count, ticket
+// zeroed before) writes phi.
+struct PoreCount {
+    unsigned long long count;
+    unsigned ticket;
+    float phi;
+};
+__global__ void porosity_kernel(const uint8_t* __restrict__ mask, long long vox_per_sample, PoreCount* pores) {
+    const uint8_t* m = mask + (long long)blockIdx.y * vox_per_sample;
+    const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
     unsigned long long c = 0;
-    for (long long i = threadIdx.x; i < vox_per_sample; i += blockDim.x) c += m[i] ? 1 : 0;
+    long long done = 0;
+    if (reinterpret_cast<uintptr_t>(m) % 16 == 0) {
+        const uint4* m4 = reinterpret_cast<const uint4*>(m);
+        for (long long i = tid; i < vox_per_sample / 16; i += step) {
+            const uint4 u = m4[i];
+            c += (__popc(__vcmpne4(u.x, 0)) + __popc(__vcmpne4(u.y, 0)) + __popc(__vcmpne4(u.z, 0)) +
+                  __popc(__vcmpne4(u.w, 0))) / 8;
+        }
+        done = vox_per_sample / 16 * 16;
+    }
+    for (long long i = done + tid; i < vox_per_sample; i += step) c += m[i] ? 1 : 0;
     for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
     __shared__ unsigned long long part[32];
     if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = c;
@@ -1196,13 +1228,20 @@ int spnn_pack_input(const uint8_t* mask, const float* optics, int B, int D, int 
     if (!mask || !optics || !x || B <= 0 || D <= 0 || H <= 0 || W <= 0) return fail(SPNN_EINVAL, "bad arguments");
     const long long vps = (long long)D * H * W, total = vps * B;
     cudaStream_t st = as_stream(stream);
-    float* phi = nullptr;
-    CU(cudaMallocAsync(reinterpret_cast<void**>(&phi), sizeof(float) * B, st));
-    porosity_kernel<<<B, 256, 0, st>>>(mask, vps, phi);
-    pack_input_kernel<<<grid_for(total), 256, 0, st>>>(mask, optics, phi, D, vps, total,
+    PoreCount* pores = nullptr;
+    CU(cudaMallocAsync(reinterpret_cast<void**>(&pores), sizeof(*pores) * B, st));
+    cudaMemsetAsync(pores, 0, sizeof(*pores) * B, st);
+    // one block per sample left the GPU idle (117 us for one 64^3 mask): about
+    // four blocks per SM over all samples, at least 16 KB of mask each
+    long long per = (4 * 152 + B - 1) / B;
+    if (per > (vps + 16383) / 16384) per = (vps + 16383) / 16384;
+    for (int b0 = 0; b0 < B; b0 += 65535)
+        porosity_kernel<<<dim3((unsigned)per, (unsigned)(B - b0 < 65535 ? B - b0 : 65535)), 256, 0, st>>>(
+            mask + (long long)b0 * vps, vps, pores + b0);
+    pack_input_kernel<<<grid_for(total), 256, 0, st>>>(mask, optics, pores, D, vps, total,
                                                         static_cast<__nv_bfloat16*>(x), H * W);
     cudaError_t e = cudaGetLastError();
-    cudaFreeAsync(phi, st);
+    cudaFreeAsync(pores, st);
     if (e != cudaSuccess) return cuda_fail(e, "pack_input launch");
     return SPNN_OK;
 }

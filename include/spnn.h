@@ -151,7 +151,7 @@ int spnn_layer_wgrad(int kind, int B, int D, int H, int W, const void* x0, int c
  * 5 (z + 1/2)/D, 6 -mu_eff (z + 1/2)/8, 7 porosity phi, 8..15 zero, where phi
  * is the sample's pore fraction and mu_eff = sqrt(3 mu_a' (mu_a' + mu_s'(1-g)))
  * the diffusion attenuation (Sec. 2.4) of the medium scaled to its solid
- * fraction, mu' = (1 - phi) mu (Eq. EMA_scaling).  Uses a B-float scratch
+ * fraction, mu' = (1 - phi) mu (Eq. EMA_scaling).  Uses a scratch of 16 B bytes
  * from the stream-ordered allocator.
  * mask: uint8 (B, D, H, W), 1 = pore;  optics: FP32 (B, 3) = (mu_s h, mu_a h, g).
  */

@@ -345,7 +345,11 @@ int rows_gemm(RowsParams& p, cudaStream_t st) {
     // all 512 columns runs alone on its SM, so its ring may use twice the budget
     p.nbuf = 2 * p.mt * p.n_tile <= 512 ? 2 : 1;
     const bool alone = tmem_cols(p.nbuf * p.mt * p.n_tile) > 256;
-    const uint32_t budget = (uint32_t)stage_budget() * (alone && g_opt_stage_kb <= 0 ? 2u : 1u);
+    // so may one of a launch of at most two tiles per SM: it runs a tile or two, so
+    // the latency of its loads shows (U-Net of batch 1: 8^3 256 -> 256 74 -> 60 us, 16^3
+    // 128 -> 128 26 -> 23 us, 256 -> 128 40 -> 35 us)
+    const bool few = n_tiles(p.g) <= 2 * 152;
+    const uint32_t budget = (alone || few) && g_opt_stage_kb <= 0 ? 200u * 1024u : (uint32_t)stage_budget();
     int S = (int)(budget / p.stage_bytes);
     p.stages = S < 2 ? 2 : (S > 8 ? 8 : S);
     p.tiles = (int)n_tiles(p.g);
@@ -897,7 +901,13 @@ __global__ void porosity_kernel(const uint8_t* __restrict__ mask, long long vox_
     if (threadIdx.x == 0) {
         unsigned long long t = 0;
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += part[w];
-        phi[blockIdx.x] = (float)((double)t / (double)vox_per_sample);
+        PoreCount* s = pores + blockIdx.y;
+        atomicAdd(&s->count, t);
+        __threadfence();
+        if (atomicAdd(&s->ticket, 1u) == gridDim.x - 1) {
+            t = atomicAdd(&s->count, 0ull);
+            s->phi = (float)((double)t / (double)vox_per_sample);
+        }
     }
 }
 
@@ -905,14 +915,14 @@ __global__ void porosity_kernel(const uint8_t* __restrict__ mask, long long vox_
 // Channel 6 is the diffusion-theory attenuation exponent -mu_eff (z + 1/2) / 8 of the
 // medium scaled to its solid fraction (mu' = (1 - phi) mu), channel 7 the porosity phi.
 __global__ void pack_input_kernel(const uint8_t* __restrict__ mask, const float* __restrict__ optics,
-                                  const float* __restrict__ phi, int D, long long vox_per_sample,
+                                  const PoreCount* __restrict__ pores, int D, long long vox_per_sample,
                                   long long total, __nv_bfloat16* __restrict__ x, int HW) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
          i += (long long)gridDim.x * blockDim.x) {
         const long long b = i / vox_per_sample;
         const int z = (int)((i % vox_per_sample) / HW);
         const float pore = mask[i] ? 1.f : 0.f;
-        const float mus = optics[3 * b], mua = optics[3 * b + 1], g = optics[3 * b + 2], ph = phi[b];
+        const float mus = optics[3 * b], mua = optics[3 * b + 1], g = optics[3 * b + 2], ph = pores[b].phi;
         const float ma = (1.f - ph) * mua, msp = (1.f - ph) * mus * (1.f - g);
         const float mu_eff = sqrtf(3.f * ma * (ma + msp));
         const float zc = z + 0.5f;

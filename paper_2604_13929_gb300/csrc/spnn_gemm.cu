@@ -147,8 +147,9 @@ __device__ __forceinline__ void tile_origin_u32(const TileGrid& g, uint32_t t, i
 // Epilogue of 16 accumulator columns of one voxel: bias, residual, ReLU or
 // ReLU-derivative mask, two 16-byte BF16 stores (channels ch0 .. ch0 + 15 at
 // off); adds the rounded outputs' dot product with head_w (if given) to head.
+// mk: the two mask words, where the caller has loaded them already.
 __device__ __forceinline__ void emit16(const EpiDest& d, const uint32_t (&v)[16], int ch0, long long off,
-                                       const float* head_w, float& head) {
+                                       const float* head_w, float& head, const uint4* mk = nullptr) {
     float f[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) f[i] = __uint_as_float(v[i]);
@@ -167,10 +168,16 @@ __device__ __forceinline__ void emit16(const EpiDest& d, const uint32_t (&v)[16]
         for (int i = 0; i < 16; ++i) f[i] = fmaxf(f[i], 0.f);
     }
     if (d.mask) {
-        float mk[16];
-        load16_planes(d.mask + off, d.plane, mk);
+        uint4 u[2];
+        u[0] = mk ? mk[0] : *reinterpret_cast<const uint4*>(d.mask + off);
+        u[1] = mk ? mk[1] : *reinterpret_cast<const uint4*>(d.mask + off + d.plane);
+        const __nv_bfloat162* m = reinterpret_cast<const __nv_bfloat162*>(u);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) f[i] = (mk[i] > 0.f) ? f[i] : 0.f;
+        for (int i = 0; i < 8; ++i) {
+            const float2 t = __bfloat1622float2(m[i]);
+            f[2 * i] = (t.x > 0.f) ? f[2 * i] : 0.f;
+            f[2 * i + 1] = (t.y > 0.f) ? f[2 * i + 1] : 0.f;
+        }
     }
     uint4 w[2];
     __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(w);
@@ -288,7 +295,7 @@ __device__ __forceinline__ void slab_issue(const SlabParams& p, uint32_t bar0, u
 // (N = 96: 56 cycles of reads for 48 of arithmetic, three taps).  Measured, rows
 // kernel -> this, batch 16 at 64^3, forward: 16 -> 32 channels 183 -> 115 us,
 // 32 -> 32 301 -> 178 us (1.30 PFLOP/s), 64 -> 32 561 -> 356 us; input gradient:
-// 32 -> 32 with mask 318 -> 227 us, 32 -> 64 349 -> 270 us (1.72 PFLOP/s).
+// 32 -> 32 with mask 318 -> 199 us, 32 -> 64 349 -> 270 us (1.72 PFLOP/s).
 // ------------------------------------------------------------------------
 template <int N, int ZC, int ZST>
 __global__ void __launch_bounds__(kSlabThreads, 1) slab_kernel(const __grid_constant__ SlabParams p) {
@@ -364,23 +371,43 @@ __global__ void __launch_bounds__(kSlabThreads, 1) slab_kernel(const __grid_cons
         const int r = q * 32 + lane;
         const int half = (warp - 2) >> 2;
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
+        const long long zstep = (long long)p.g.H * p.g.W;
+        // ReLU masks of a plane, loaded a plane (the first: an accumulator wait)
+        // ahead (64^3 32 -> 32, batch 16: 199 us; 228 where each chunk waits for its own)
+        auto load_masks = [&](long long vox, uint4 (&mk)[N / 8]) {
+#pragma unroll
+            for (int n0 = 0; n0 < N; n0 += 16) {
+                const EpiDest& d = (n0 < p.split) ? p.d[0] : p.d[1];
+                if (d.mask == nullptr || d.out == nullptr) continue;
+                const __nv_bfloat16* src = d.mask + ((n0 - d.col0) >> 3) * d.plane + vox * 8;
+                mk[n0 / 8] = *reinterpret_cast<const uint4*>(src);
+                mk[n0 / 8 + 1] = *reinterpret_cast<const uint4*>(src + d.plane);
+            }
+        };
+        const bool masks = p.d[0].mask != nullptr || p.d[1].mask != nullptr;
         uint32_t it = 0;
         for (int t = blockIdx.x; t < p.tiles; t += gridDim.x, ++it) {
             const uint32_t buf = it & 1u, use = it >> 1;
+            int x0, y0, z0, b0;
+            tile_origin_u32(p.g, (uint32_t)t, x0, y0, z0, b0);
+            const int x = x0 + r % p.g.bx, y = y0 + r / p.g.bx;
+            // two warps per quarter of the rows: even and odd planes
+            long long vox = (((long long)b0 * p.g.D + z0 + half) * p.g.H + y) * p.g.W + x;
+            uint4 mk[N / 8], next[N / 8];
+            if (masks) load_masks(vox, next);
             if (!__all_sync(0xffffffffu, mbar_wait(acc_full + 8u * buf, use & 1u, kWaitLimitNs))) {
                 if (lane == 0) atomicOr(p.err, ERR_TIMEOUT);
                 break;
             }
             tc_fence_after();
-            int x0, y0, z0, b0;
-            tile_origin_u32(p.g, (uint32_t)t, x0, y0, z0, b0);
-            const int x = x0 + r % p.g.bx, y = y0 + r / p.g.bx;
-            // two warps per quarter of the rows: even and odd planes
-            const long long zstep = (long long)p.g.H * p.g.W;
-            long long vox = (((long long)b0 * p.g.D + z0 + half) * p.g.H + y) * p.g.W + x;
             for (int z = half; z < p.zp; z += 2, vox += 2 * zstep) {
                 const uint32_t col = tmem + buf * acc_cols + lane_base + (uint32_t)(z * N);
                 float head = 0.f;
+                if (masks) {
+#pragma unroll
+                    for (int i = 0; i < N / 8; ++i) mk[i] = next[i];
+                    if (z + 2 < p.zp) load_masks(vox + 2 * zstep, next);
+                }
 #pragma unroll
                 for (int n0 = 0; n0 < N; n0 += 16) {
                     uint32_t v[16];
@@ -389,7 +416,8 @@ __global__ void __launch_bounds__(kSlabThreads, 1) slab_kernel(const __grid_cons
                     const EpiDest& d = (n0 < p.split) ? p.d[0] : p.d[1];
                     if (d.out == nullptr) continue;
                     const int ch0 = n0 - d.col0;
-                    emit16(d, v, ch0, (ch0 >> 3) * d.plane + vox * 8, p.head_out ? p.head_w : nullptr, head);
+                    emit16(d, v, ch0, (ch0 >> 3) * d.plane + vox * 8, p.head_out ? p.head_w : nullptr, head,
+                           &mk[n0 / 8]);
                 }
                 if (p.head_out) p.head_out[vox] = head + *p.head_b;
             }

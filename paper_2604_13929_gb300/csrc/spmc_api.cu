@@ -629,6 +629,15 @@ int sp_mc_get_option(const sp_mc_t *h, int key, double *value) {
     }
 }
 
+// Steps per pass worth taking for the FP32 kernel.  A lane whose photon interacts
+// waits for the end of the pass; with an interaction every 1.5 / (mu_s (1 - phi))
+// steps or so, a pass of 8 wastes more than a second event phase costs below
+// about 16 (16 masks of 64^3 36.1 -> 34.1 ms and 256^3 phi 0.70 profiles 58.5 ->
+// 57.0 ms with 4; 256^3 phi 0.90, 30 steps, 40.6 -> 40.8 ms and keeps 8).
+static int pass_cap(const sp_mc *h) {
+    return h->mus * (1.0 - h->porosity) * 16.0 > 1.5 ? 4 : 64;
+}
+
 // Runs that record photons and volumes whose voxel addresses need more than
 // 32 bits take the FP32 kernel's general builds.
 static bool wide_build(const sp_mc *h) { return h->n_rec > 0 || h->n_field > 0xffffffffull; }
@@ -690,7 +699,7 @@ static int launch_run(sp_mc *h, u64 n_photons, u64 seed, u64 pid_begin, const u6
     p.iter_limit = iter_limit(h);
     p.compact_k = h->compact_k;
     p.mirror = h->mirror;
-    p.steps_per_pass = h->steps_per_pass;
+    p.steps_per_pass = std::min(h->steps_per_pass, pass_cap(h));
     p.bin_mul = h->bin_mul;
     p.bin_exact = h->bin_exact;
     fill_f32(h, p.s_max, p.f32, p.hg_iso, p.small_x, p.plain);
@@ -1330,6 +1339,7 @@ extern "C" int sp_mc_batch_run(sp_mc_batch_t *b, const uint64_t *n_photons, uint
             t.iter_limit = lim > 0xffffffffull ? 0xffffffffu : (u32)lim;
             fill_f32(h, path_cap(h), t.f32, t.hg_iso, t.small_x, t.plain);
             t.mirror = h->mirror;
+            t.pass_cap = pass_cap(h);
             CUDA_TRY(cudaMemsetAsync(&h->d_tal->next, 0, sizeof(u64), s));
         }
         group_problems(b);

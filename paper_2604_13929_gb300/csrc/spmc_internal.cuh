@@ -108,6 +108,7 @@ struct BatchProblem {
     int group, group_end;
     u32 iter_limit;
     int hg_iso, small_x, plain, mirror;
+    int pass_cap;                  // most steps per pass worth taking for these optics
     TransportParams::F32 f32;
 };
 

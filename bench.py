@@ -62,16 +62,16 @@ SFU_INTERACT, SFU_PHOTON = 10, 1
 ISSUE_PER_SM_CLK = 4          # warp instructions per SM per clock (4 schedulers)
 SFU_PER_SM_CLK = 16           # XU lane-operations per SM per clock
 # DRAM bytes (read + write) per photon of the transport kernel from one ncu capture
-# (a 2e6-photon launch of this workload: 3.593e9 B read + 2.897e10 B written),
+# (a 2e6-photon launch of this workload: 3.603e9 B read + 2.890e10 B written),
 # valid only for the kernel source it was taken on.
-TRAFFIC_CAPTURE = {"kernel_sha256_prefix": "3e0680a07320195d", "dram_bytes_per_photon": 16283.4,
+TRAFFIC_CAPTURE = {"kernel_sha256_prefix": "caff656deea1a694", "dram_bytes_per_photon": 16249.3,
                    "source": "profiles/transport_kernel_256cubed_phi090.md"}
 # Hardware fractions of peak of the transport kernel from the same ncu capture
 # (smsp__issue_active, sm__inst_executed_pipe_xu, lts__d_atomic_input_cycles_active),
 # reported only while the kernel source matches the capture.
-NCU_FRACTIONS = {"kernel_sha256_prefix": "3e0680a07320195d", "issue_slots": 0.5831,
-                 "sfu_xu_pipe": 0.0164, "l2_atomic_unit": 0.1924, "warps_active": 0.3668,
-                 "l2_red_hit_rate": 0.6543, "registers_per_thread": 72,
+NCU_FRACTIONS = {"kernel_sha256_prefix": "caff656deea1a694", "issue_slots": 0.5080,
+                 "sfu_xu_pipe": 0.0315, "l2_atomic_unit": 0.2550, "warps_active": 0.3706,
+                 "l2_red_hit_rate": 0.6543, "registers_per_thread": 71,
                  "source": "profiles/transport_kernel_256cubed_phi090.md"}
 
 

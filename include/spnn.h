@@ -70,11 +70,14 @@ int spnn_status(void* stream);
  *                           stacked along y, sharing one halo box and weight copy
  *   SPNN_OPT_CONV_PLANES    8-channel chunk planes per conv3 K-step (2, 4)
  *   SPNN_OPT_STAGE_KB       shared-memory budget of the stage ring in KB (<= 220)
- *   SPNN_OPT_WGRAD_HALO     1 (default): conv3 weight gradients with at most 32
- *                           output channels on halo K-steps (one input box and
- *                           three shifted output-gradient boxes per x-run);
- *                           2: wherever they fit (up to 80 output channels);
- *                           0: always the per-tap kernel
+ *   SPNN_OPT_WGRAD_HALO     1 (default): conv3 weight gradients on row windows
+ *                           (16, 32 or a multiple of 64 output channels, rows of
+ *                           8 voxels or more), else with at most 32 output
+ *                           channels on halo K-steps (one input box and three
+ *                           shifted output-gradient boxes per x-run), else the
+ *                           per-tap kernel; 2: halo K-steps wherever they fit
+ *                           (up to 80 output channels); 0: always the per-tap
+ *                           kernel
  *   SPNN_OPT_CONV_FULL_HALO 1: conv3 forward / input gradient on 8 x 16 tiles whose
  *                           one box per plane block serves all 27 taps, where it
  *                           fits; 0 (default): one box per x-shift
@@ -87,7 +90,9 @@ int spnn_status(void* stream);
  *                           squared error by exp(target) over its sample's mean
  *                           of exp(target) (targets are log fluences); 0
  *                           (default): unweighted
- * Settings that do not fit a layer fall back to the automatic choice.
+ * Settings that do not fit a layer fall back to the automatic choice.  conv3
+ * forward and input-gradient GEMMs of 16, 32 or 64 output columns walk along z
+ * (same results) unless one of the first two or the full-halo option is set.
  */
 #define SPNN_OPT_CONV_SUBTILES 1
 #define SPNN_OPT_CONV_PLANES 2

@@ -92,10 +92,10 @@ enum sp_option {
                                 the compacted event phase); 0 the generic
                                 template kernel (same photons, same method) */
     SP_OPT_STEPS_PER_PASS = 17,/* streamlined kernel: voxel steps a lane
-                                takes at most per pass of its warp, [1, 64]
-                                (8; 4 at most with optics where photons
-                                interact within about 16 steps); results
-                                do not depend on it                        */
+                                takes at most per pass of its warp, [1, 64];
+                                until it is set 8, or 4 with optics where
+                                photons interact within about 16 steps;
+                                results do not depend on it                */
     SP_OPT_BATCH_CHUNK = 18   /* batched one-launch mode, streamlined kernel:
                                 photons per warp claim, [32, 2^24] (128);
                                 results do not depend on it                */

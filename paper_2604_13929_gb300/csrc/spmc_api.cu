@@ -21,6 +21,7 @@
 
 #include "spmc.h"
 #include "spmc_internal.cuh"
+#include "spmc_plan.h"
 
 using namespace spmc;
 
@@ -74,7 +75,7 @@ struct sp_mc {
     int compact_k = 8;
     int mirror = 0;         // lateral faces: 0 periodic, 1 mirrors
     int variant = 1;        // FP32 kernel: 0 generic template, 1 streamlined
-    int steps_per_pass = 8; // streamlined FP32 kernel: voxel steps per warp pass
+    int steps_per_pass = 0; // streamlined FP32 kernel: voxel steps per warp pass; 0 automatic
     u32 bin_mul = 0;        // depth bin by multiply-high, when exact for this nz
     int bin_exact = 0;
     // device memory
@@ -624,18 +625,9 @@ int sp_mc_get_option(const sp_mc_t *h, int key, double *value) {
     case SP_OPT_COMPACT: *value = h->compact_k; return SP_OK;
     case SP_OPT_LATERAL_BC: *value = h->mirror; return SP_OK;
     case SP_OPT_KERNEL: *value = h->variant; return SP_OK;
-    case SP_OPT_STEPS_PER_PASS: *value = h->steps_per_pass; return SP_OK;
+    case SP_OPT_STEPS_PER_PASS: *value = h->steps_per_pass ? h->steps_per_pass : kPassSteps; return SP_OK;
     default: return fail(SP_EINVAL, "unknown option %d", key);
     }
-}
-
-// Steps per pass worth taking for the FP32 kernel.  A lane whose photon interacts
-// waits for the end of the pass; with an interaction every 1.5 / (mu_s (1 - phi))
-// steps or so, a pass of 8 wastes more than a second event phase costs below
-// about 16 (16 masks of 64^3 36.1 -> 34.1 ms and 256^3 phi 0.70 profiles 58.5 ->
-// 57.0 ms with 4; 256^3 phi 0.90, 30 steps, 40.6 -> 40.8 ms and keeps 8).
-static int pass_cap(const sp_mc *h) {
-    return h->mus * (1.0 - h->porosity) * 16.0 > 1.5 ? 4 : 64;
 }
 
 // Runs that record photons and volumes whose voxel addresses need more than
@@ -646,7 +638,6 @@ static bool wide_build(const sp_mc *h) { return h->n_rec > 0 || h->n_field > 0xf
 // (or from *pid_begin_dev when it is set), stream-ordered and capturable.
 static int launch_run(sp_mc *h, u64 n_photons, u64 seed, u64 pid_begin, const u64 *pid_begin_dev,
                       cudaStream_t s) {
-
     const u64 n_bricks = (u64)h->nbx * h->nby * h->nbz;
     int smem_bricks = h->smem_bricks_opt;
     if (smem_bricks < 0) smem_bricks = (int)std::min<u64>(n_bricks, 12288);   // auto: 96 KiB
@@ -699,7 +690,7 @@ static int launch_run(sp_mc *h, u64 n_photons, u64 seed, u64 pid_begin, const u6
     p.iter_limit = iter_limit(h);
     p.compact_k = h->compact_k;
     p.mirror = h->mirror;
-    p.steps_per_pass = std::min(h->steps_per_pass, pass_cap(h));
+    p.steps_per_pass = pass_steps(h->steps_per_pass, h->mus, h->porosity);
     p.bin_mul = h->bin_mul;
     p.bin_exact = h->bin_exact;
     fill_f32(h, p.s_max, p.f32, p.hg_iso, p.small_x, p.plain);
@@ -983,7 +974,10 @@ extern "C" int sp_mc_simulate_noalloc(const uint8_t *d_mask, int nx, int ny, int
     const double porosity = (double)n_pore / ((double)nx * (double)ny * (double)nz);
 
     // Default options of a fresh handle, profile-only tally (no voxel field);
-    // the launch constants come from the same helpers as sp_mc_run's.
+    // the launch constants come from the same helpers as sp_mc_run's, but for the
+    // pass length: the few photons of such a call wait for the longest history, which
+    // shorter passes only slow down (20000 photons, 64^3 phi 0.70: 8 steps 1.13 ms,
+    // 4 steps 1.17 ms).
     sp_mc tmp;
     tmp.nx = nx; tmp.ny = ny; tmp.nz = nz;
     tmp.mus = mu_s * voxel_h; tmp.mua = mu_a * voxel_h; tmp.g = g;
@@ -1012,7 +1006,7 @@ extern "C" int sp_mc_simulate_noalloc(const uint8_t *d_mask, int nx, int ny, int
     p.iter_limit = iter_limit(&tmp);
     p.compact_k = tmp.compact_k;
     p.mirror = 0;
-    p.steps_per_pass = tmp.steps_per_pass;
+    p.steps_per_pass = pass_steps(kPassSteps, tmp.mus, tmp.porosity);
     p.bin_mul = tmp.bin_mul;
     p.bin_exact = tmp.bin_exact;
     fill_f32(&tmp, p.s_max, p.f32, p.hg_iso, p.small_x, p.plain);
@@ -1059,7 +1053,7 @@ struct sp_mc_batch {
     BatchProblem *d_table = nullptr;
     u64 *d_next = nullptr;
     int threads = 128, blocks_per_sm = 0, compact_k = 8, use_graph = 1, mode = 0;
-    int variant = 1, steps_per_pass = 8;   // one-launch kernel and its steps per pass
+    int variant = 1, steps_per_pass = 0;   // one-launch kernel and its steps per pass (0 automatic)
     u32 chunk = 128;                       // photons per warp claim (streamlined kernel): small
                                            // claims keep the problems in flight, and so the
                                            // voxel fields written, few (L2)
@@ -1201,7 +1195,7 @@ extern "C" int sp_mc_batch_get_option(const sp_mc_batch_t *b, int key, double *v
     case SP_OPT_BATCH_MODE: *value = b->mode; return SP_OK;
     case SP_OPT_BATCH_CHUNK: *value = b->chunk; return SP_OK;
     case SP_OPT_KERNEL: *value = b->variant; return SP_OK;
-    case SP_OPT_STEPS_PER_PASS: *value = b->steps_per_pass; return SP_OK;
+    case SP_OPT_STEPS_PER_PASS: *value = b->steps_per_pass ? b->steps_per_pass : kPassSteps; return SP_OK;
     default: return sp_mc_get_option(b->h[0], key, value);
     }
 }
@@ -1339,7 +1333,7 @@ extern "C" int sp_mc_batch_run(sp_mc_batch_t *b, const uint64_t *n_photons, uint
             t.iter_limit = lim > 0xffffffffull ? 0xffffffffu : (u32)lim;
             fill_f32(h, path_cap(h), t.f32, t.hg_iso, t.small_x, t.plain);
             t.mirror = h->mirror;
-            t.pass_cap = pass_cap(h);
+            t.pass_steps = pass_steps(0, h->mus, h->porosity);
             CUDA_TRY(cudaMemsetAsync(&h->d_tal->next, 0, sizeof(u64), s));
         }
         group_problems(b);
@@ -1421,10 +1415,10 @@ extern "C" int sp_mc_batch_autotune(sp_mc_batch_t *b, const uint64_t *n_photons,
     CUDA_TRY(cudaEventCreate(&e0));
     CUDA_TRY(cudaEventCreate(&e1));
     // one-launch candidates: threads per CTA, all or half the resident CTAs,
-    // compaction threshold and (streamlined kernel) steps per pass
+    // compaction threshold and (streamlined kernel) steps per pass: automatic or long
     const int threads_c[] = {64, 128, 256};
     const int compact_c[] = {4, 8, 12, 16};
-    const int spp_c[] = {8, 16};
+    const int spp_c[] = {0, 16};
     double best = -1.0;
     int best_t = b->threads, best_b = b->blocks_per_sm, best_k = b->compact_k, best_mode = 0;
     int best_spp = b->steps_per_pass;

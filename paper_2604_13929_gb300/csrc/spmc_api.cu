@@ -645,13 +645,13 @@ static int launch_run(sp_mc *h, u64 n_photons, u64 seed, u64 pid_begin, const u6
     const bool f64 = h->precision == 64;
     const bool field = h->field != 0;
     const size_t extra = f64 ? 0 : smem_f32(field, h->variant, h->threads);
-    constexpr size_t kMaxSmem = 227 * 1024;
-    // the FP32 kernel's own shared memory comes out of a slab that would
-    // otherwise fill an SM's (staging more or fewer bricks changes no result)
-    if (extra && (size_t)smem_bricks * sizeof(u64) + 4352 <= kMaxSmem)
-        smem_bricks = (int)std::min<size_t>((size_t)smem_bricks, (kMaxSmem - extra) / sizeof(u64));
-    const size_t smem = (size_t)smem_bricks * sizeof(u64) + extra;
     const bool wide = wide_build(h);
+    int per_sm = 0;
+    if (extra && smem_bricks) {
+        CUDA_TRY(occupancy_f32(field, h->mirror != 0, h->variant, wide, h->threads, extra, &per_sm));
+        smem_bricks = staged_bricks(smem_bricks, extra, per_sm);
+    }
+    const size_t smem = (size_t)smem_bricks * sizeof(u64) + extra;
     if (smem > 48 * 1024) {
         CUDA_TRY(cudaFuncSetAttribute(f64 ? kernel_f64(field, h->mirror != 0)
                                           : kernel_f32(field, h->mirror != 0, h->variant, wide),
@@ -659,7 +659,6 @@ static int launch_run(sp_mc *h, u64 n_photons, u64 seed, u64 pid_begin, const u6
     }
     int blocks = h->blocks_opt;
     if (blocks <= 0) {
-        int per_sm = 0;
         CUDA_TRY(f64 ? occupancy_f64(field, h->mirror != 0, h->threads, smem, &per_sm)
                      : occupancy_f32(field, h->mirror != 0, h->variant, wide, h->threads, smem, &per_sm));
         if (per_sm < 1) return fail(SP_ECUDA, "transport kernel cannot be resident with %zu B smem", smem);

@@ -70,3 +70,13 @@ def test_batched_pass_lengths_agree(spmc, length):
         for i, problem in enumerate(problems):
             ref = _run(spmc, problem, n[i], steps_per_pass=1, path_cap=55.7)
             _assert_same(ref, (b.tallies(i), b.raw_field(i)), (i, length))
+
+
+@pytest.mark.parametrize("field", [1, 0])
+@pytest.mark.parametrize("threads", [64, 256])
+def test_staged_bricks_agree(spmc, field, threads):
+    """Staging the entry slab of the mask, as many bricks as fit, changes no result."""
+    problem = (inputs.random_mask((96, 92, 100), 0.9, 5), 0.3, 0.01, 0.6)
+    base = _run(spmc, problem, 20000, tally_field=field, threads=threads)
+    for bricks in (-1, 1, 2048, 12288, 28000):
+        _assert_same(base, _run(spmc, problem, 20000, tally_field=field, threads=threads, smem_bricks=bricks), bricks)

@@ -10,6 +10,7 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 SOURCE = r"""
 #include "spmc_plan.h"
 extern "C" int pass_steps(int option, double mus, double porosity) { return spmc::pass_steps(option, mus, porosity); }
+extern "C" int staged_bricks(int want, size_t own, int resident) { return spmc::staged_bricks(want, own, resident); }
 """
 
 
@@ -24,6 +25,7 @@ def rules(tmp_path_factory):
     subprocess.run([cxx, "-std=c++17", "-shared", "-fPIC", f"-I{CSRC}", "-o", str(lib), str(src)], check=True)
     r = ctypes.CDLL(str(lib))
     r.pass_steps.argtypes = [ctypes.c_int, ctypes.c_double, ctypes.c_double]
+    r.staged_bricks.argtypes = [ctypes.c_int, ctypes.c_size_t, ctypes.c_int]
     return r
 
 
@@ -37,3 +39,24 @@ def test_automatic_pass_length_follows_the_optics(rules):
     assert rules.pass_steps(0, 0.5, 0.70) == 4          # an interaction every 10 steps
     assert rules.pass_steps(0, 0.5, 0.90) == 8          # every 30
     assert rules.pass_steps(0, 0.0, 0.5) == 8
+
+
+@pytest.mark.parametrize("own", [4352, 20736, 21760, 42000])
+@pytest.mark.parametrize("resident", [3, 4, 8])
+@pytest.mark.parametrize("want", [0, 1, 512, 2048, 5000, 8192, 12288, 20000, 28512])
+def test_staged_bricks_keep_the_resident_ctas(rules, want, own, resident):
+    """The slab shrinks by the kernel's own shared memory instead of costing a CTA per SM."""
+    per_sm, per_cta, reserved, bare = 228 * 1024, 227 * 1024, 1024, 4352
+    n = rules.staged_bricks(want, own, resident)
+    before = max(1, min(resident, per_sm // (8 * want + bare + reserved)))
+    assert 0 <= n <= want
+    assert 8 * n + own <= per_cta
+    if n:
+        assert min(resident, per_sm // (8 * n + own + reserved)) >= before
+        assert n == want or 8 * (n + 1) + own > min(per_cta, per_sm // before - reserved)
+
+
+def test_staged_bricks_at_scratch_limits(rules):
+    assert rules.staged_bricks(28513, 21760, 4) == 28513      # over 227 KB beside the tallies: refused by the launch
+    assert rules.staged_bricks(20000, 0, 4) == 20000          # a kernel without shared memory of its own
+    assert rules.staged_bricks(-1, 21760, 4) == -1

@@ -13,6 +13,7 @@
 
 #include "spnn.h"
 #include "spnn_internal.cuh"
+#include "spnn_plan.h"
 #include "spnn_umma.cuh"
 
 using namespace spnn;
@@ -342,14 +343,15 @@ int rows_gemm(RowsParams& p, cudaStream_t st) {
     rows_geometry(p);
     if (p.mt < 1) p.mt = 1;
     // two accumulator buffers where they fit in TMEM; a CTA whose buffers take
-    // all 512 columns runs alone on its SM, so its ring may use twice the budget
+    // more than half of its columns runs alone on its SM
     p.nbuf = 2 * p.mt * p.n_tile <= 512 ? 2 : 1;
     const bool alone = tmem_cols(p.nbuf * p.mt * p.n_tile) > 256;
-    // so may one of a launch of at most two tiles per SM: it runs a tile or two, so
-    // the latency of its loads shows (U-Net of batch 1: 8^3 256 -> 256 74 -> 60 us, 16^3
-    // 128 -> 128 26 -> 23 us, 256 -> 128 40 -> 35 us)
-    const bool few = n_tiles(p.g) <= 2 * 152;
-    const uint32_t budget = (alone || few) && g_opt_stage_kb <= 0 ? 200u * 1024u : (uint32_t)stage_budget();
+    const int grid_n = p.n_total / p.n_tile;
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return cuda_fail(e, "device attributes");
+    const uint32_t budget = ring_budget(n_tiles(p.g), grid_n, sms, p.scatter_up, alone, g_opt_stage_kb);
     int S = (int)(budget / p.stage_bytes);
     p.stages = S < 2 ? 2 : (S > 8 ? 8 : S);
     p.tiles = (int)n_tiles(p.g);
@@ -360,11 +362,10 @@ int rows_gemm(RowsParams& p, cudaStream_t st) {
     p.idesc = idesc_bf16(128, p.n_tile, 0, 0);
     p.err = err_ptr();
     if (!p.err) return fail(SPNN_ECUDA, "no device");
-    const int grid_n = p.n_total / p.n_tile;
     if (grid_n > kMaxGridN) return fail(SPNN_EINVAL, "GEMM N %d: more than %d N tiles", p.n_total, kMaxGridN);
     static std::atomic<unsigned> ctr_next{0};   // launches may come from several host threads
     void* ctr = nullptr;
-    cudaError_t e = cudaGetSymbolAddress(&ctr, g_tile_ctr);
+    e = cudaGetSymbolAddress(&ctr, g_tile_ctr);
     if (e != cudaSuccess) return cuda_fail(e, "tile counters");
     p.tile_ctr = static_cast<int*>(ctr) + (size_t)(ctr_next.fetch_add(1) % kCtrSlots) * kMaxGridN;
     e = cudaMemsetAsync(p.tile_ctr, 0, sizeof(int) * grid_n, st);

@@ -9,8 +9,12 @@ import pytest
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2604_13929_gb300", "csrc")
 SOURCE = r"""
 #include "spmc_plan.h"
+#include "spnn_plan.h"
 extern "C" int pass_steps(int option, double mus, double porosity) { return spmc::pass_steps(option, mus, porosity); }
 extern "C" int staged_bricks(int want, size_t own, int resident) { return spmc::staged_bricks(want, own, resident); }
+extern "C" unsigned ring_budget(long long tiles, int grid_n, int sms, int scatter, int alone, int option_kb) {
+    return spnn::ring_budget(tiles, grid_n, sms, scatter, alone, option_kb);
+}
 """
 
 
@@ -26,6 +30,8 @@ def rules(tmp_path_factory):
     r = ctypes.CDLL(str(lib))
     r.pass_steps.argtypes = [ctypes.c_int, ctypes.c_double, ctypes.c_double]
     r.staged_bricks.argtypes = [ctypes.c_int, ctypes.c_size_t, ctypes.c_int]
+    r.ring_budget.argtypes = [ctypes.c_longlong] + [ctypes.c_int] * 5
+    r.ring_budget.restype = ctypes.c_uint
     return r
 
 
@@ -60,3 +66,16 @@ def test_staged_bricks_at_scratch_limits(rules):
     assert rules.staged_bricks(28513, 21760, 4) == 28513      # over 227 KB beside the tallies: refused by the launch
     assert rules.staged_bricks(20000, 0, 4) == 20000          # a kernel without shared memory of its own
     assert rules.staged_bricks(-1, 21760, 4) == -1
+
+
+@pytest.mark.parametrize("tiles,grid_n,scatter,alone,kb", [
+    (4, 1, 0, 0, 200), (32, 1, 0, 0, 200), (304, 1, 0, 0, 200), (305, 1, 0, 0, 110), (152, 2, 0, 0, 200),
+    (153, 2, 0, 0, 110),
+    # N tiles count: up 256 -> 128 from 8^3 at batch 64 is 256 boxes x 8 N tiles; scatter
+    # epilogues keep two CTAs per SM however few tiles there are
+    (256, 8, 0, 0, 110), (256, 8, 1, 0, 110), (4, 8, 1, 0, 110), (32, 4, 1, 0, 110),
+    (4, 1, 0, 1, 220), (5000, 1, 0, 1, 220), (5000, 1, 1, 1, 220),
+])
+def test_ring_budget_counts_output_tiles(rules, tiles, grid_n, scatter, alone, kb):
+    assert rules.ring_budget(tiles, grid_n, 152, scatter, alone, 0) == kb * 1024
+    assert rules.ring_budget(tiles, grid_n, 152, scatter, alone, 90) == 90 * 1024

@@ -143,7 +143,7 @@ int spnn_layer_dgrad(int kind, int B, int D, int H, int W, const void* dy, int c
 /*
  * Weight and bias gradients of one layer, ADDED (FP32 atomics) into
  * dw[taps][c0 + c1][cout] and db[cout] (db may be NULL).  x0, x1 as in
- * spnn_layer_forward; dy as in spnn_layer_dgrad.
+ * spnn_layer_forward; dy as in spnn_layer_dgrad.  cout <= 256.
  */
 int spnn_layer_wgrad(int kind, int B, int D, int H, int W, const void* x0, int c0, const void* x1, int c1,
                      const void* dy, int cout, float* dw, float* db, void* stream);

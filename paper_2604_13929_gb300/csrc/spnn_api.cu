@@ -723,7 +723,8 @@ int wgrad_halo(int B, int D, int H, int W, const void* x0, int c0, const void* x
 int wgrad_rows(int B, int D, int H, int W, const void* x0, int c0, const void* x1, int c1, const void* dy,
                int cout, float* dw, float* db, cudaStream_t st) {
     const int kc0 = c0 / 8, kc1 = c1 / 8, kc = kc0 + kc1;
-    if (cout != 16 && cout != 32 && cout % 64) return 1;
+    // (more than 256 output channels: refused by the per-tap kernel's planner, as for every layer)
+    if ((cout != 16 && cout != 32 && cout % 64) || cout > 256) return 1;
     WgradRowsParams p;
     memset(&p, 0, sizeof p);
     p.nc = cout < 64 ? cout : 64;

@@ -77,3 +77,19 @@ def test_batched_builds_equal_single_runs(spmc, mirror):
             _assert_same(b.tallies(i), sim.tallies(check=False), i)
             assert np.array_equal(b.raw_field(i), sim.raw_field())
             sim.close()
+
+
+def test_path_moment_sums_carry(spmc):
+    """Straight flights through a pore column of 11863283 voxels: two photons of a lane
+    already overflow 64 bits of the second moment, all lanes of a block end together, and
+    the sums must be the exact 128-bit integers."""
+    nz, n = 11863283, 256 * 3
+    sim = spmc.Simulation(np.ones((nz, 1, 1), dtype=np.uint8), 0.5, 0.005, 0.7, tally_field=0, blocks=1)
+    sim.run(n, 3)
+    t = sim.tallies()
+    path = np.float32(nz)
+    words = lambda v: [v % 2 ** 64, v >> 64]                                      # noqa: E731
+    assert t["exit_T"] == n
+    assert [int(x) for x in t["raw_sum_wP"]] == words(n * int(path) * 2 ** 32)
+    assert [int(x) for x in t["raw_sum_wP2"]] == words(n * int(path * path) * 2 ** 16)
+    sim.close()

@@ -250,28 +250,6 @@ bool conv_tiling_with(int opt_mt, int opt_planes, int B, int D, int H, int W, in
     return false;
 }
 
-// Output planes per box of the z-walk (0: the layer does not fit it).  It takes
-// layers of 16, 32 or 64 output channels (3 n <= 256 columns in one MMA) whose
-// weights stay resident in half of shared memory; above that the z-taps no
-// longer share the A reads that bound them, or the ring gets too short.  Of
-// the depths that fit two buffers into TMEM it takes the cheapest: an MMA of
-// N columns costs about max(N / 2, (128 + N) / 4) cycles (tensor rate, operand
-// reads of 128 bytes a cycle), and the boxes go over the SMs in whole rounds.
-int slab_depth(const TileGrid& g, int n, int kc_total, int sms) {
-    if ((n != 16 && n != 32 && n != 64) || g.bz != 1 || g.bb != 1 || 27 * kc_total * n * 16 > 112 * 1024) return 0;
-    auto mma = [&](int k) { const int N = k * n; return N / 2 > (128 + N) / 4 ? N / 2 : (128 + N) / 4; };
-    const long long columns = (long long)g.nx * g.ny * g.B;
-    int best = 0;
-    long long best_cost = 0;
-    for (int zp = 2; zp <= 16 && zp <= g.D; zp *= 2) {
-        if (2 * zp * n > 512) break;
-        const long long rounds = (columns * (g.D / zp) + sms - 1) / sms;
-        const long long cost = rounds * ((zp - 2) * mma(3) + 2 * mma(2) + 2 * mma(1));
-        if (!best || cost <= best_cost) best = zp, best_cost = cost;
-    }
-    return best;
-}
-
 // conv3 GEMM by the z-walk; p holds the rows GEMM of the same layer (grid of
 // one-plane tiles of 128 mt voxels, planes per K-step, destinations).  Returns
 // 1 when the layer does not fit.
@@ -284,8 +262,11 @@ int slab_gemm(const RowsParams& p, const void* x0, int c0, const void* x1, int c
     SlabParams q;
     memset(&q, 0, sizeof q);
     if (!make_grid(kRows, p.g.B, p.g.D, p.g.H, p.g.W, &q.g)) return 1;
-    q.zp = slab_depth(q.g, p.n_total, p.kc_total, sms);
-    if (!q.zp) return 1;
+    if (q.g.bz != 1 || q.g.bb != 1) return 1;
+    const SlabShape shape = slab_shape(q.g.bx, q.g.by, (long long)q.g.nx * q.g.ny * q.g.B, q.g.D, p.n_total,
+                                       p.kc_total, sms);
+    if (!shape.zp) return 1;
+    q.zp = shape.zp;
     q.g.bz = q.zp;
     q.g.nz = q.g.D / q.zp;
     q.n = p.n_total;
@@ -293,13 +274,9 @@ int slab_gemm(const RowsParams& p, const void* x0, int c0, const void* x1, int c
     q.kc0 = p.kc0;
     q.wpack = p.wpack;
     q.tiles = (int)n_tiles(q.g);
-    q.w_bytes = 27u * p.kc_total * q.n * 16u;
-    // one CTA per SM (its accumulators take up to 512 TMEM columns)
-    const int zc = slab_zc(q.zp);
-    q.stage_bytes = (uint32_t)(2 * zc * (q.g.by + 2) * q.g.bx * 16);
-    q.stages = (int)((220u * 1024u - q.w_bytes) / q.stage_bytes);
-    if (q.stages > 8) q.stages = 8;
-    if (q.stages < 3 || q.stage_bytes % 128) return 1;
+    q.w_bytes = shape.w_bytes;
+    q.stage_bytes = shape.stage_bytes;
+    q.stages = shape.stages;
     q.split = p.split;
     q.d[0] = p.d[0];
     q.d[1] = p.d[1];
@@ -315,7 +292,7 @@ int slab_gemm(const RowsParams& p, const void* x0, int c0, const void* x1, int c
         if (!c) continue;
         cuuint64_t dims[5] = {8ull * q.g.W, (cuuint64_t)q.g.H, (cuuint64_t)q.g.D, (cuuint64_t)q.g.B, (cuuint64_t)(c / 8)};
         cuuint64_t strides[4] = {row, row * q.g.H, row * q.g.H * q.g.D, row * q.g.H * q.g.D * q.g.B};
-        cuuint32_t box[5] = {8u * q.g.bx, (cuuint32_t)q.g.by + 2, (cuuint32_t)zc, 1, 2};
+        cuuint32_t box[5] = {8u * q.g.bx, (cuuint32_t)q.g.by + 2, (cuuint32_t)slab_zc(q.zp), 1, 2};
         int rc = encode(&q.maps[i], x, dims, strides, box);
         if (rc) return rc;
     }

@@ -207,9 +207,6 @@ cudaError_t launch_wgrad_rows(const WgradRowsParams& p, int nm, dim3 grid, size_
 // Persistent launch: min(tiles, persistent x SMs x resident CTAs) x grid_n CTAs.
 constexpr int kMaxGridN = 16;               // N tiles of one rows GEMM (claim counters per launch)
 cudaError_t launch_rows(const RowsParams& p, int grid_n, size_t smem, cudaStream_t s);
-// Input planes per stage of the z-walk: the most that divide zp + 2 into at
-// least two stages of at most six.
-__host__ __device__ constexpr int slab_zc(int zp) { return zp == 16 ? 6 : (zp == 8 ? 5 : (zp == 4 ? 3 : 2)); }
 constexpr int kSlabEpiWarps = 8;            // two per quarter of the accumulator's rows
 constexpr int kSlabThreads = 64 + 32 * kSlabEpiWarps;
 cudaError_t launch_slab(const SlabParams& p, int grid, size_t smem, cudaStream_t s);

@@ -15,6 +15,9 @@ extern "C" int staged_bricks(int want, size_t own, int resident) { return spmc::
 extern "C" unsigned ring_budget(long long tiles, int grid_n, int sms, int scatter, int alone, int option_kb) {
     return spnn::ring_budget(tiles, grid_n, sms, scatter, alone, option_kb);
 }
+extern "C" int slab_depth(int bx, int by, long long columns, int D, int n, int kc_total, int sms) {
+    return spnn::slab_shape(bx, by, columns, D, n, kc_total, sms).zp;
+}
 """
 
 
@@ -31,6 +34,7 @@ def rules(tmp_path_factory):
     r.pass_steps.argtypes = [ctypes.c_int, ctypes.c_double, ctypes.c_double]
     r.staged_bricks.argtypes = [ctypes.c_int, ctypes.c_size_t, ctypes.c_int]
     r.ring_budget.argtypes = [ctypes.c_longlong] + [ctypes.c_int] * 5
+    r.slab_depth.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_longlong] + [ctypes.c_int] * 4
     r.ring_budget.restype = ctypes.c_uint
     return r
 
@@ -79,3 +83,31 @@ def test_staged_bricks_at_scratch_limits(rules):
 def test_ring_budget_counts_output_tiles(rules, tiles, grid_n, scatter, alone, kb):
     assert rules.ring_budget(tiles, grid_n, 152, scatter, alone, 0) == kb * 1024
     assert rules.ring_budget(tiles, grid_n, 152, scatter, alone, 90) == 90 * 1024
+
+
+def _slab(rules, B, D, H, W, cin, cout):
+    """Box depth of the z-walk on 152 SMs and boxes per CTA."""
+    bx = min(W, 32)
+    by = 128 // bx
+    assert H >= by                                            # one-plane tiles
+    columns = (W // bx) * (H // by) * B
+    zp = rules.slab_depth(bx, by, columns, D, cout, cin // 8, 152)
+    return zp, columns * (D // zp) / 152 if zp else 0
+
+
+def test_slab_cases_reach_every_depth_with_reused_buffers(rules):
+    from test_gpu_surrogate_slab_depths import CASES
+    reached = set()
+    for *shape, depth in CASES:
+        zp, boxes = _slab(rules, *shape)
+        assert zp == depth, shape
+        if boxes > 2:
+            reached.add((shape[-1], zp))
+    assert reached == {(16, 2), (16, 4), (16, 8), (16, 16), (32, 2), (32, 4), (32, 8), (64, 2), (64, 4)}
+
+
+@pytest.mark.parametrize("n,cin,fits", [(16, 16, True), (32, 64, True), (32, 80, False), (64, 32, True), (64, 48, False),
+                                        (48, 16, False), (128, 16, False), (8, 16, False)])
+def test_slab_takes_only_what_fits(rules, n, cin, fits):
+    assert (rules.slab_depth(32, 4, 64, 32, n, cin // 8, 152) > 0) == fits
+    assert rules.slab_depth(32, 4, 64, 1, n, cin // 8, 152) == 0          # no depth to walk

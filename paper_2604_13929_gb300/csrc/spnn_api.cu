@@ -851,8 +851,8 @@ cudaStream_t as_stream(void* s) { return static_cast<cudaStream_t>(s); }
 
 // --------------------------------------------------------- data kernels --
 // Pore fraction of each sample's mask: gridDim.x blocks per sample, 16 mask
-// bytes per load where aligned; the sample's last block to finish (count, ticket
-// zeroed before) writes phi.
+// bytes per load where aligned; the sample's last block to finish writes phi (with
+// more than one, count and ticket are zeroed before).
 struct PoreCount {
     unsigned long long count;
     unsigned ticket;
@@ -881,12 +881,14 @@ __global__ void porosity_kernel(const uint8_t* __restrict__ mask, long long vox_
         unsigned long long t = 0;
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += part[w];
         PoreCount* s = pores + blockIdx.y;
-        atomicAdd(&s->count, t);
-        __threadfence();
-        if (atomicAdd(&s->ticket, 1u) == gridDim.x - 1) {
-            t = atomicAdd(&s->count, 0ull);
-            s->phi = (float)((double)t / (double)vox_per_sample);
+        bool last = gridDim.x == 1;
+        if (!last) {
+            atomicAdd(&s->count, t);
+            __threadfence();
+            last = atomicAdd(&s->ticket, 1u) == gridDim.x - 1;
+            if (last) t = atomicAdd(&s->count, 0ull);
         }
+        if (last) s->phi = (float)((double)t / (double)vox_per_sample);
     }
 }
 
@@ -1219,11 +1221,11 @@ int spnn_pack_input(const uint8_t* mask, const float* optics, int B, int D, int 
     cudaStream_t st = as_stream(stream);
     PoreCount* pores = nullptr;
     CU(cudaMallocAsync(reinterpret_cast<void**>(&pores), sizeof(*pores) * B, st));
-    cudaMemsetAsync(pores, 0, sizeof(*pores) * B, st);
     // one block per sample left the GPU idle (117 us for one 64^3 mask): about
     // four blocks per SM over all samples, at least 16 KB of mask each
     long long per = (4 * 152 + B - 1) / B;
     if (per > (vps + 16383) / 16384) per = (vps + 16383) / 16384;
+    if (per > 1) cudaMemsetAsync(pores, 0, sizeof(*pores) * B, st);
     for (int b0 = 0; b0 < B; b0 += 65535)
         porosity_kernel<<<dim3((unsigned)per, (unsigned)(B - b0 < 65535 ? B - b0 : 65535)), 256, 0, st>>>(
             mask + (long long)b0 * vps, vps, pores + b0);

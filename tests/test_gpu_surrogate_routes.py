@@ -91,3 +91,21 @@ def test_rows_gemm_conv3_is_independent_of_its_grid(S, B, D, H, W, c0, c1, cout)
         S.spnn_status()
         outs.append(y)
     assert all(torch.equal(y, outs[0]) for y in outs[1:]) and float(outs[0].float().abs().sum()) > 0
+
+
+@pytest.mark.parametrize("B,n,skew", [(1, 16, 0), (64, 16, 0), (3, 24, 0), (1, 32, 0), (5, 32, 1), (700, 8, 3), (2, 64, 5)])
+def test_pack_input_porosity(S, B, n, skew):
+    """Channel 7 is each sample's pore fraction, counted by one block per sample or several,
+    from masks at any byte offset."""
+    gen = torch.Generator(device="cuda").manual_seed(n + B)
+    flat = torch.zeros(B * n ** 3 + skew, dtype=torch.uint8, device="cuda")
+    mask = flat[skew:].view(B, n, n, n)
+    level = torch.linspace(0.0, 1.0, B, device="cuda").view(B, 1, 1, 1)
+    mask.copy_((torch.rand((B, n, n, n), generator=gen, device="cuda") < level).to(torch.uint8))
+    optics = torch.tensor([[0.5, 0.005, 0.7]] * B, device="cuda")
+    for _ in range(2):                                   # the second call may find the first one's scratch
+        x = S.planes_empty(B, n, n, n, 16)
+        S.spnn_pack_input(mask, optics, x)
+        phi = S.from_planes(x)[..., 7]
+        want = mask.view(B, -1).double().mean(dim=1).to(torch.float32).to(torch.bfloat16)
+        assert torch.equal(phi.reshape(B, -1), want[:, None].expand(B, n ** 3))

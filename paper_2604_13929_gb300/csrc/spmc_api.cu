@@ -601,7 +601,7 @@ int sp_mc_set_option(sp_mc_t *h, int key, double value) {
         if (value != 0 && value != 1) return fail(SP_EINVAL, "kernel variant must be 0 or 1");
         h->variant = (int)value; return SP_OK;
     case SP_OPT_STEPS_PER_PASS:
-        if (value < 1 || value > 64) return fail(SP_EINVAL, "steps per pass must be in [1, 64]");
+        if (value < 1 || value > kPassStepsMax) return fail(SP_EINVAL, "steps per pass must be in [1, 64]");
         h->steps_per_pass = (int)value; return SP_OK;
     default: return fail(SP_EINVAL, "unknown option %d", key);
     }
@@ -1060,6 +1060,7 @@ struct sp_mc_batch {
     bool table_valid = false;              // device table matches table[]
     std::vector<u64> cfg_n;                // configuration of the device table / graph
     u64 cfg_seed = 0;
+    int cfg_spp = 0;
     cudaStream_t cap = nullptr;            // private stream for graph capture
     cudaGraphExec_t exec = nullptr;
     int graph_threads = 0, graph_blocks = 0, graph_compact = 0, graph_mode = 0, graph_variant = 0,
@@ -1160,7 +1161,7 @@ extern "C" int sp_mc_batch_set_option(sp_mc_batch_t *b, int key, double value) {
         // the one-launch kernel's own setting, and every problem's for mode 1
         if (key == SP_OPT_KERNEL && value != 0 && value != 1)
             return fail(SP_EINVAL, "kernel variant must be 0 or 1");
-        if (key == SP_OPT_STEPS_PER_PASS && (value < 1 || value > 64))
+        if (key == SP_OPT_STEPS_PER_PASS && (value < 1 || value > kPassStepsMax))
             return fail(SP_EINVAL, "steps per pass must be in [1, 64]");
         if (key == SP_OPT_KERNEL) b->variant = (int)value; else b->steps_per_pass = (int)value;
         for (sp_mc *h : b->h) {
@@ -1245,7 +1246,7 @@ static int batch_launch(sp_mc_batch *b, u64 total, cudaStream_t s) {
     bp.key0 = (u32)b->cfg_seed;
     bp.key1 = (u32)(b->cfg_seed >> 32);
     bp.compact_k = b->compact_k;
-    bp.steps_per_pass = b->steps_per_pass;
+    bp.steps_per_pass = b->steps_per_pass ? b->steps_per_pass : kPassSteps;
     CUDA_TRY(cudaMemsetAsync(b->d_next, 0, b->n * sizeof(u64), s));
     CUDA_TRY(launch_transport_batch(bp, b->variant, b->any_mirror, per_sm * b->sm_count, b->threads, s));
     batch_advance_kernel<<<(b->n + 127) / 128, 128, 0, s>>>(b->d_table, b->n);
@@ -1310,7 +1311,8 @@ extern "C" int sp_mc_batch_run(sp_mc_batch_t *b, const uint64_t *n_photons, uint
         if (rc) return rc;
     }
     const std::vector<u64> want(n_photons, n_photons + b->n);
-    const bool same_cfg = b->table_valid && want == b->cfg_n && seed == b->cfg_seed;
+    const bool same_cfg = b->table_valid && want == b->cfg_n && seed == b->cfg_seed &&
+                          b->cfg_spp == b->steps_per_pass;
     if (!same_cfg) {
         // (re)build the device table from the handles' photon counters
         u64 offset = 0;
@@ -1332,7 +1334,7 @@ extern "C" int sp_mc_batch_run(sp_mc_batch_t *b, const uint64_t *n_photons, uint
             t.iter_limit = lim > 0xffffffffull ? 0xffffffffu : (u32)lim;
             fill_f32(h, path_cap(h), t.f32, t.hg_iso, t.small_x, t.plain);
             t.mirror = h->mirror;
-            t.pass_steps = pass_steps(0, h->mus, h->porosity);
+            t.pass_cap = b->steps_per_pass ? kPassStepsMax : pass_steps(0, h->mus, h->porosity);
             CUDA_TRY(cudaMemsetAsync(&h->d_tal->next, 0, sizeof(u64), s));
         }
         group_problems(b);
@@ -1341,6 +1343,7 @@ extern "C" int sp_mc_batch_run(sp_mc_batch_t *b, const uint64_t *n_photons, uint
         CUDA_TRY(cudaStreamSynchronize(s));     // the host table may change after return
         b->cfg_n = want;
         b->cfg_seed = seed;
+        b->cfg_spp = b->steps_per_pass;
         b->table_valid = true;
         if (b->exec) { cudaGraphExecDestroy(b->exec); b->exec = nullptr; }
     }

@@ -108,7 +108,7 @@ struct BatchProblem {
     int group, group_end;
     u32 iter_limit;
     int hg_iso, small_x, plain, mirror;
-    int pass_steps;                // automatic steps per pass of these optics
+    int pass_cap;                  // most steps per pass: the automatic length of these optics, 64 where one was set
     TransportParams::F32 f32;
 };
 
@@ -121,7 +121,7 @@ struct BatchParams {
                                     // (streamlined kernel), or the first for all photons
     u32 key0, key1;                 // Philox key = seed (shared by all problems)
     int compact_k;
-    int steps_per_pass;             // 0: each problem's own
+    int steps_per_pass;
 };
 
 // Launch choices of the FP32 path beyond TransportParams: which kernel.

@@ -80,3 +80,20 @@ def test_staged_bricks_agree(spmc, field, threads):
     base = _run(spmc, problem, 20000, tally_field=field, threads=threads)
     for bricks in (-1, 1, 2048, 12288, 28000):
         _assert_same(base, _run(spmc, problem, 20000, tally_field=field, threads=threads, smem_bricks=bricks), bricks)
+
+
+def test_pass_length_change_between_graph_replays(spmc):
+    """Setting the pass length rebuilds the problem table and the captured graph; photon ids go on."""
+    problems = [(inputs.random_mask((40, 24, 24), 0.95, 1), 0.3, 0.01, 0.6),
+                (inputs.random_mask((20, 16, 12), 0.6, 2), 1.5, 0.02, 0.2)]
+    n = [9000, 5000]
+    with spmc.Batch(problems, graph=1) as b:
+        assert b.get_option("steps_per_pass") == 8
+        for length in (None, None, 29, 29, 1):
+            if length:
+                b.set_option("steps_per_pass", length)
+                assert b.get_option("steps_per_pass") == length
+            b.run(n, 29)
+        for i, problem in enumerate(problems):
+            ref = _run(spmc, problem, 5 * n[i], steps_per_pass=1)
+            _assert_same(ref, (b.tallies(i), b.raw_field(i)), i)

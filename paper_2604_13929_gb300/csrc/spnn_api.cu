@@ -328,7 +328,7 @@ int rows_gemm(RowsParams& p, cudaStream_t st) {
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return cuda_fail(e, "device attributes");
-    const uint32_t budget = ring_budget(n_tiles(p.g), grid_n, sms, p.scatter_up, alone, g_opt_stage_kb);
+    const uint32_t budget = ring_budget(n_tiles(p.g), grid_n, p.ksteps, sms, p.scatter_up, alone, g_opt_stage_kb);
     int S = (int)(budget / p.stage_bytes);
     p.stages = S < 2 ? 2 : (S > 8 ? 8 : S);
     p.tiles = (int)n_tiles(p.g);

@@ -14,11 +14,19 @@ namespace spnn {
 // 30 -> 26 us, 256 -> 128 46 -> 38 us).  Not so with a scatter epilogue (up forward,
 // down input gradient), which bounds those layers: up 8^3 256 -> 128 took 83 us at
 // batch 64 with half an SM and 114 us with a whole one, down 16^3 128 -> 256 input
-// gradients 110 and 144 us.
-inline uint32_t ring_budget(long long tiles, int grid_n, int sms, bool scatter, bool alone, int option_kb) {
+// gradients 110 and 144 us.  But for one case: with two N tiles, the first one's CTAs
+// (up to a box each) take the SMs' two slots before the second's, and with between
+// 5/3 and 2 boxes per SM they leave it so few that those do nearly all its tiles.  If
+// the tiles are short (one or two K-steps), one CTA per SM, so that the N tiles follow
+// one another, is faster: up 32^3 64 -> 32 at batch 1 (256 boxes) 33 us against 29 us,
+// 288 boxes 37 and 33 us; 248 boxes 30 and 32 us, 304 29 and 35 us.
+inline uint32_t ring_budget(long long tiles, int grid_n, int ksteps, int sms, bool scatter, bool alone,
+                            int option_kb) {
     if (option_kb > 0) return (uint32_t)option_kb * 1024u;
     if (alone) return 220u * 1024u;
-    return !scatter && tiles * grid_n <= 2ll * sms ? 200u * 1024u : 110u * 1024u;
+    const bool whole = scatter ? grid_n == 2 && ksteps <= 2 && 3 * tiles >= 5ll * sms && tiles < 2ll * sms
+                               : tiles * grid_n <= 2ll * sms;
+    return (whole ? 200u : 110u) * 1024u;
 }
 
 // Input planes per stage of the z-walk: the most that divide zp + 2 into at

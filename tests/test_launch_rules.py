@@ -12,8 +12,8 @@ SOURCE = r"""
 #include "spnn_plan.h"
 extern "C" int pass_steps(int option, double mus, double porosity) { return spmc::pass_steps(option, mus, porosity); }
 extern "C" int staged_bricks(int want, size_t own, int resident) { return spmc::staged_bricks(want, own, resident); }
-extern "C" unsigned ring_budget(long long tiles, int grid_n, int sms, int scatter, int alone, int option_kb) {
-    return spnn::ring_budget(tiles, grid_n, sms, scatter, alone, option_kb);
+extern "C" unsigned ring_budget(long long tiles, int grid_n, int ksteps, int sms, int scatter, int alone, int option_kb) {
+    return spnn::ring_budget(tiles, grid_n, ksteps, sms, scatter, alone, option_kb);
 }
 extern "C" int slab_depth(int bx, int by, long long columns, int D, int n, int kc_total, int sms) {
     return spnn::slab_shape(bx, by, columns, D, n, kc_total, sms).zp;
@@ -33,7 +33,7 @@ def rules(tmp_path_factory):
     r = ctypes.CDLL(str(lib))
     r.pass_steps.argtypes = [ctypes.c_int, ctypes.c_double, ctypes.c_double]
     r.staged_bricks.argtypes = [ctypes.c_int, ctypes.c_size_t, ctypes.c_int]
-    r.ring_budget.argtypes = [ctypes.c_longlong] + [ctypes.c_int] * 5
+    r.ring_budget.argtypes = [ctypes.c_longlong] + [ctypes.c_int] * 6
     r.slab_depth.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_longlong] + [ctypes.c_int] * 4
     r.ring_budget.restype = ctypes.c_uint
     return r
@@ -72,17 +72,21 @@ def test_staged_bricks_at_scratch_limits(rules):
     assert rules.staged_bricks(-1, 21760, 4) == -1
 
 
-@pytest.mark.parametrize("tiles,grid_n,scatter,alone,kb", [
-    (4, 1, 0, 0, 200), (32, 1, 0, 0, 200), (304, 1, 0, 0, 200), (305, 1, 0, 0, 110), (152, 2, 0, 0, 200),
-    (153, 2, 0, 0, 110),
+@pytest.mark.parametrize("tiles,grid_n,ksteps,scatter,alone,kb", [
+    (4, 1, 9, 0, 0, 200), (32, 1, 9, 0, 0, 200), (304, 1, 9, 0, 0, 200), (305, 1, 9, 0, 0, 110), (152, 2, 9, 0, 0, 200),
+    (153, 2, 1, 0, 0, 110),
     # N tiles count: up 256 -> 128 from 8^3 at batch 64 is 256 boxes x 8 N tiles; scatter
-    # epilogues keep two CTAs per SM however few tiles there are
-    (256, 8, 0, 0, 110), (256, 8, 1, 0, 110), (4, 8, 1, 0, 110), (32, 4, 1, 0, 110),
-    (4, 1, 0, 1, 220), (5000, 1, 0, 1, 220), (5000, 1, 1, 1, 220),
+    # epilogues keep two CTAs per SM however few tiles there are ...
+    (256, 8, 4, 0, 0, 110), (256, 8, 4, 1, 0, 110), (4, 8, 4, 1, 0, 110), (32, 4, 2, 1, 0, 110), (128, 2, 1, 1, 0, 110),
+    (256, 4, 1, 1, 0, 110), (256, 1, 1, 1, 0, 110),
+    # ... except where the first of two N tiles would leave the second few CTAs
+    (253, 2, 1, 1, 0, 110), (254, 2, 1, 1, 0, 200), (256, 2, 2, 1, 0, 200), (303, 2, 1, 1, 0, 200),
+    (304, 2, 1, 1, 0, 110), (256, 2, 3, 1, 0, 110),
+    (4, 1, 9, 0, 1, 220), (5000, 1, 9, 0, 1, 220), (5000, 1, 1, 1, 1, 220),
 ])
-def test_ring_budget_counts_output_tiles(rules, tiles, grid_n, scatter, alone, kb):
-    assert rules.ring_budget(tiles, grid_n, 152, scatter, alone, 0) == kb * 1024
-    assert rules.ring_budget(tiles, grid_n, 152, scatter, alone, 90) == 90 * 1024
+def test_ring_budget_counts_output_tiles(rules, tiles, grid_n, ksteps, scatter, alone, kb):
+    assert rules.ring_budget(tiles, grid_n, ksteps, 152, scatter, alone, 0) == kb * 1024
+    assert rules.ring_budget(tiles, grid_n, ksteps, 152, scatter, alone, 90) == 90 * 1024
 
 
 def _slab(rules, B, D, H, W, cin, cout):

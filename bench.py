@@ -62,15 +62,15 @@ SFU_INTERACT, SFU_PHOTON = 10, 1
 ISSUE_PER_SM_CLK = 4          # warp instructions per SM per clock (4 schedulers)
 SFU_PER_SM_CLK = 16           # XU lane-operations per SM per clock
 # DRAM bytes (read + write) per photon of the transport kernel from one ncu capture
-# (a 2e6-photon launch of this workload: 3.603e9 B read + 2.890e10 B written),
+# (a 2e6-photon launch of this workload: 3.603e9 B read + 2.889e10 B written),
 # valid only for the kernel source it was taken on.
-TRAFFIC_CAPTURE = {"kernel_sha256_prefix": "caff656deea1a694", "dram_bytes_per_photon": 16249.3,
+TRAFFIC_CAPTURE = {"kernel_sha256_prefix": "c7b8640c42d05a5c", "dram_bytes_per_photon": 16248.5,
                    "source": "profiles/transport_kernel_256cubed_phi090.md"}
 # Hardware fractions of peak of the transport kernel from the same ncu capture
 # (smsp__issue_active, sm__inst_executed_pipe_xu, lts__d_atomic_input_cycles_active),
 # reported only while the kernel source matches the capture.
-NCU_FRACTIONS = {"kernel_sha256_prefix": "caff656deea1a694", "issue_slots": 0.5080,
-                 "sfu_xu_pipe": 0.0315, "l2_atomic_unit": 0.2550, "warps_active": 0.3706,
+NCU_FRACTIONS = {"kernel_sha256_prefix": "c7b8640c42d05a5c", "issue_slots": 0.5073,
+                 "sfu_xu_pipe": 0.0315, "l2_atomic_unit": 0.2569, "warps_active": 0.3705,
                  "l2_red_hit_rate": 0.6543, "registers_per_thread": 71,
                  "source": "profiles/transport_kernel_256cubed_phi090.md"}
 
@@ -538,7 +538,7 @@ def surrogate_bench(torch, args):
             "data_seconds": data_s, "mc_photons_per_s": mc_photons_per_s,
             "roofline": {"bound": "tensor", "achieved": achieved, "peak": peaks["bf16_tflops_sustained"],
                          "unit": "TFLOP/s", "frac": achieved / peaks["bf16_tflops_sustained"], "traffic": None,
-                         "kernel": "spnn rows_kernel, all 20 forward layers", "flop_per_field": fl,
+                         "kernel": "spnn rows_kernel and slab_kernel, all 20 forward layers", "flop_per_field": fl,
                          "peak_source": "MEASURED_PEAKS.json bf16_tflops_sustained (of measured)"},
             "gpu_launches": 22 * 10, "clocks": clk.summary()}
     print(json.dumps(line), flush=True)
@@ -738,7 +738,7 @@ def main():
                 "unit": "Gwarp-inst/s", "frac": achieved / peak, "traffic": traffic,
                 "traffic_note": "DRAM read+write bytes per launch, ncu capture scaled by the "
                                 "photon count (null if the kernel source changed since)",
-                "kernel": ("spmc::transport_f32_kernel<true,false>" if variant == 1
+                "kernel": ("spmc::transport_f32_kernel<true,false,false,false>" if variant == 1
                            else "spmc::transport_kernel<float,true,false,false>"),
                 "kernel_sha256_prefix": sha,
                 "ops_per_unit": {"voxel_step": OPS_STEP, "solid_step_extra": OPS_SOLID_EXTRA,
@@ -757,7 +757,7 @@ def main():
                 "ncu_fractions": (NCU_FRACTIONS if NCU_FRACTIONS
                                   and NCU_FRACTIONS.get("kernel_sha256_prefix") == sha else None)}
 
-    # measured ceiling of the step pattern: straight rays through an all-pore
+    # measured rate of the step pattern: straight rays through an all-pore
     # 256^3 volume, with and without one Q32.32 RED per step into a 256^3 field
     ceil_red = spmc.sp_mc_probe_step_ceiling(N_VOX, True)["steps_per_s"]
     ceil_nored = spmc.sp_mc_probe_step_ceiling(N_VOX, False)["steps_per_s"]
@@ -765,10 +765,11 @@ def main():
     roofline["step_ceiling"] = {
         "with_field_red_steps_per_s": ceil_red, "without_red_steps_per_s": ceil_nored,
         "with_field_red_240cubed_steps_per_s": ceil_fit,
-        "frac_of_red_ceiling": value * steps_per_photon / ceil_red,
+        "ratio_to_red_probe": value * steps_per_photon / ceil_red,
         "note": "sp_mc_probe_step_ceiling: the kernel's traversal and tally memory pattern "
                 "with no physics; the 256^3 Q32.32 field (134 MB) is past the L2 knee, a 240^3 "
-                "field (111 MB) is not"}
+                "field (111 MB) is not. Its rays move through the field in step, photons do not, "
+                "so the transport may exceed it: a rate to compare with, not a ceiling"}
 
     # end to end through the C ABI with host buffers: upload + pack the host
     # mask, transport, normalise, copy the results back
